@@ -97,8 +97,8 @@ enum {
   MOND_OPT_TIMING = 4,    /* value 1: bracket every launch with CUDA events (see mond_pm_kernel_stats) */
   MOND_OPT_PIPELINED = 5, /* value 1 (default): y/z passes stream tiles with TMA through a two-stage ring;
                              0: one tile per CTA with plain loads (same results) */
-  MOND_OPT_CHUNK = 6,     /* particles per deposit/gather work item: a power of two in 256..4096
-                             (default 1024; same results) */
+  MOND_OPT_CHUNK = 6,     /* particles per deposit/gather work item at most: a power of two in 256..4096
+                             (default 1024; a small system's items are smaller; same results) */
   MOND_OPT_GATHER = 7,    /* force at the particles. 0 (default): Eq. gi, the ball sum at each particle.
                              1 or 3: the mesh-interpolating gather -- the final pass of a solve (n_iter >= 1)
                              also multiplies the acceleration spectrum by the smoothing spectrum, so that

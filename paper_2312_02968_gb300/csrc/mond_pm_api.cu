@@ -43,10 +43,7 @@ struct Workspace {
   float* kp;
   uint32_t* lut;
   uint32_t* ball;
-  int32_t* ball_lin;   // per tap: linear mesh offset of an interior ball
-  int32_t* ball_hlin;  // per tap: linear offset inside a tile plus its reach
-  int32_t* rows;       // rows of the ball, two orders (deposit, gather) of nrows each:
-                       // [k] tile offset of the row centre, [nrows + k] dy | dz << 8 | L << 16
+  int32_t* rows;       // rows of the ball, dy | dz << 8 | L << 16 (shifted by r)
   uint64_t* dep;
   float2* W;         // 3 spectral planes
   float2* A;         // 4 spectral planes
@@ -62,8 +59,10 @@ struct Workspace {
   int* cstart;       // n^3 + 2 sorted starts
   int* bsum;         // scan block sums
   int* tile_start;
-  int* chunk_start;
+  int4* items;       // work items of the deposit and the gather (parts::Work)
 };
+
+constexpr int MIN_CHUNK = 64;  // particles of a work item at least (but for the remainders)
 
 bool size_supported(int n) {
   switch (n) {
@@ -82,6 +81,12 @@ int ball_reach(double sigma) {
   return r;
 }
 
+// Entries of the work-item list: full items of 64 particles or more, and a
+// remainder per tile that is not sparse.
+int work_cap(int ntile, int64_t maxp) {
+  return (int)(maxp / MIN_CHUNK + std::min<int64_t>(ntile, maxp / parts::SPARSE) + 1);
+}
+
 // Layout of the workspace; when base is null only the size is computed.
 size_t carve(int n, int r, int nb, int64_t maxp, char* base, Workspace* w) {
   size_t off = 0;
@@ -94,7 +99,7 @@ size_t carve(int n, int r, int nb, int64_t maxp, char* base, Workspace* w) {
   const int64_t plane = (int64_t)n * n * (n / 2 + 2);
   const int ntx = n / parts::TILE;
   const int ntile = ntx * ntx * ntx;
-  const int lw = 2 * r + 1;
+  const int lw = parts::axis_pitch(r);
   Workspace t{};
   t.status = (uint32_t*)take(256);
   t.red = (double*)take(sizeof(double) * (256 + dens::MAX_BINS));
@@ -106,9 +111,7 @@ size_t carve(int n, int r, int nb, int64_t maxp, char* base, Workspace* w) {
   t.kp = (float*)take(sizeof(float) * n);
   t.lut = (uint32_t*)take(sizeof(uint32_t) * 65537 * lw);
   t.ball = (uint32_t*)take(sizeof(uint32_t) * nb);
-  t.ball_lin = (int32_t*)take(sizeof(int32_t) * nb);
-  t.ball_hlin = (int32_t*)take(sizeof(int32_t) * nb);
-  t.rows = (int32_t*)take(sizeof(int32_t) * 4 * (2 * r + 1) * (2 * r + 1));
+  t.rows = (int32_t*)take(sizeof(int32_t) * (2 * r + 1) * (2 * r + 1));
   t.dep = (uint64_t*)take(sizeof(uint64_t) * n3);
   t.W = (float2*)take(sizeof(float2) * 3 * plane);
   t.A = (float2*)take(sizeof(float2) * 4 * plane);
@@ -124,7 +127,7 @@ size_t carve(int n, int r, int nb, int64_t maxp, char* base, Workspace* w) {
   t.cstart = (int*)take(sizeof(int) * (n3 + 2));
   t.bsum = (int*)take(sizeof(int) * ((n3 + 1) / parts::SCAN_B + 2));
   t.tile_start = (int*)take(sizeof(int) * (ntile + 2));
-  t.chunk_start = (int*)take(sizeof(int) * (ntile + 2));
+  t.items = (int4*)take(sizeof(int4) * work_cap(ntile, maxp));
   if (w) *w = t;
   return off;
 }
@@ -332,6 +335,7 @@ struct mond_pm {
   cudaEvent_t ev_copy0 = nullptr, ev_vel = nullptr;
   int vel_wait = 0;
   bool capturing = false;
+  uint32_t dep_max_sum = 1;  // parts::DepArgs::max_sum for the axis table
   int chunk = parts::CHUNK;  // particles per deposit/gather work item
   // captured step (MOND_OPT_USE_GRAPH): the launch sequence of one
   // mond_pm_step for the key below, replayed with one cudaGraphLaunch
@@ -676,10 +680,24 @@ int read_status(mond_pm* h) {
   return MOND_OK;
 }
 
-// CTAs of the persistent deposit and gather (work items from a counter).
-int persistent_ctas(const mond_pm* h) {
-  const int g = h->sms * 4;
+// CTAs of the persistent deposit and gather (work from counters): as many as
+// are resident, per_sm a kernel's CTAs per SM, and no more than particles.
+int persistent_ctas(const mond_pm* h, int per_sm) {
+  const int g = (int)std::max<int64_t>(1, std::min<int64_t>(h->N, (int64_t)h->sms * per_sm));
   return (h->grid_cap > 0 && h->grid_cap < g) ? h->grid_cap : g;
+}
+
+// Particles per work item: the option's value, halved while the particles
+// would make fewer than four full items per SM (down to 64: an item's fixed
+// cost, staging and flushing its tile, is that of about 30 particles).
+int chunk_of(const mond_pm* h) {
+  int c = h->chunk;
+  while (c > MIN_CHUNK && h->N < (int64_t)c * 4 * h->sms) c >>= 1;
+  return c;
+}
+
+parts::Work work_of(const mond_pm* h) {
+  return {h->w.items, work_cap(h->ntile, h->maxp), h->w.key, h->w.counters + 4};
 }
 
 int do_bin(mond_pm* h) {
@@ -697,8 +715,8 @@ int do_bin(mond_pm* h) {
   b.cstart = h->w.cstart;
   b.bsum = h->w.bsum;
   b.tile_start = h->w.tile_start;
-  b.chunk_start = h->w.chunk_start;
-  b.chunk = h->chunk;
+  b.work = work_of(h);
+  b.chunk = chunk_of(h);
   b.perm = h->w.perm;
   b.status = h->w.status;
   const int64_t M = h->n3 + 1;
@@ -731,29 +749,11 @@ int do_bin(mond_pm* h) {
   CK(cudaGetLastError());
   h->count_dirty = false;
   {
-    // work items per tile, then their exclusive scan in place (chunk_start[T] = total)
     Timed tm(h, KC_BIN, 16.0 * h->ntile);
-    const int T = h->ntile, nbt = (T + parts::SCAN_B - 1) / parts::SCAN_B;
-    parts::k_tile_counts<<<(T + 255) / 256, 256, 0, h->st>>>(b);
-    parts::k_scan_reduce<<<nbt, 1024, 0, h->st>>>(h->w.chunk_start, T, h->w.bsum);
-    parts::k_scan_blocks<<<1, 1024, 0, h->st>>>(h->w.bsum, nbt);
-    parts::k_scan_apply<<<nbt, 1024, 0, h->st>>>(h->w.chunk_start, T, h->w.bsum, h->w.chunk_start);
-    h->launches += 3;  // the Timed scope counts one of the four launches
+    parts::k_tile_work<<<(h->ntile + 255) / 256, 256, 0, h->st>>>(b);
   }
   CK(cudaGetLastError());
   return MOND_OK;
-}
-
-// taps per lane kept in registers: the smallest instantiated width covering
-// the ball, 0 when it is too wide (the kernels then read the taps from shared
-// memory)
-size_t dep_smem(mond_pm* h) {
-  int hw = parts::TILE + 2 * h->r;
-  return sizeof(uint32_t) * 3 * (size_t)hw * hw * (hw + 1) + sizeof(uint32_t) * 3 * h->nb;
-}
-size_t gat_smem(mond_pm* h) {
-  int hw = parts::TILE + 2 * h->r;
-  return sizeof(float) * 4 * (size_t)hw * hw * (hw + 1);
 }
 
 template <typename K>
@@ -766,6 +766,8 @@ cudaError_t launch_smem(K kern, unsigned grid, unsigned block, size_t sm, cudaSt
 
 int do_deposit(mond_pm* h) {
   CK(cudaMemsetAsync(h->w.dep, 0, sizeof(uint64_t) * h->n3, h->st));
+  // work counters: [0, 1] deposit, [2, 3] gather, [4..6] entries of the work list
+  CK(cudaMemsetAsync(h->w.counters, 0, 7 * sizeof(int), h->st));
   int rc = do_bin(h);
   if (rc) return rc;
   parts::DepArgs d{};
@@ -778,26 +780,23 @@ int do_deposit(mond_pm* h) {
   d.off = h->off;
   d.mass = h->mass;
   d.perm = h->w.perm;
-  d.tile_start = h->w.tile_start;
-  d.chunk_start = h->w.chunk_start;
-  d.chunk = h->chunk;
+  d.work = work_of(h);
   d.lut = h->w.lut;
   d.ball = h->w.ball;
-  d.ball_lin = h->w.ball_lin;
-  d.ball_hlin = h->w.ball_hlin;
   d.rows = h->w.rows;
   d.nrows = h->nrows;
   d.dep = h->w.dep;
   d.kacc = h->kacc;
+  d.max_sum = h->dep_max_sum;
   d.work_counter = h->w.counters;
-  CK(cudaMemsetAsync(h->w.counters, 0, sizeof(int), h->st));
-  size_t sm = dep_smem(h);
   {
     // algorithmic bytes: particle reads (perm, cell, offset, mass) and one int64 write per touched cell
     Timed tm(h, KC_DEPOSIT, 32.0 * h->N + 8.0 * h->n3);
+    const bool wide = 16.0 * h->sigma * h->sigma == (double)((h->r + 1) * (h->r + 1));
     switch (h->r) {
 #define DEPOSIT_R(R) \
-  case R: CK(launch_smem(parts::k_deposit<R>, persistent_ctas(h), parts::DEP_NT, sm, h->st, &d)); break;
+  case R: CK(launch_smem(wide ? parts::k_deposit<R, true> : parts::k_deposit<R, false>, persistent_ctas(h, parts::dep_ctas(R)), parts::DEP_NT, \
+                         parts::dep_smem_bytes<R>(), h->st, &d)); break;
       DEPOSIT_R(2) DEPOSIT_R(3) DEPOSIT_R(4) DEPOSIT_R(5) DEPOSIT_R(6) DEPOSIT_R(7)
 #undef DEPOSIT_R
       default: return fail(h, MOND_EINVAL, "no deposit for reach %d", h->r);
@@ -823,12 +822,10 @@ int do_gather(mond_pm* h, float* g_out, double dt, int kick, int drift) {
   g.vel = h->vel;
   g.perm = h->w.perm;
   g.tile_start = h->w.tile_start;
-  g.chunk_start = h->w.chunk_start;
-  g.chunk = h->chunk;
+  g.work = work_of(h);
   g.acc = h->w.acc;
   g.ball = h->w.ball;
-  g.ball_hlin = h->w.ball_hlin;
-  g.rows = h->w.rows + 2 * h->nrows;  // the gather's order
+  g.rows = h->w.rows;
   g.nrows = h->nrows;
   g.g_out = g_out;
   g.dt = (float)dt;
@@ -837,7 +834,7 @@ int do_gather(mond_pm* h, float* g_out, double dt, int kick, int drift) {
   g.do_drift = drift;
   g.inv2s2 = (float)(1.0 / (2.0 * h->sigma * h->sigma));
   g.gnorm = (float)(1.0 / (h->sigma * sqrt(2.0 * M_PI)));
-  g.work_counter = h->w.counters + 1;
+  g.work_counter = h->w.counters + 2;
   g.status = h->w.status;
   if ((h->gather_mode != 0) != h->acc_smoothed)
     return fail(h, MOND_ESTATE, h->gather_mode ? "the interpolating gather needs a solve with n_iter >= 1 made with "
@@ -852,14 +849,13 @@ int do_gather(mond_pm* h, float* g_out, double dt, int kick, int drift) {
     CK(cudaGetLastError());
     return MOND_OK;
   }
-  CK(cudaMemsetAsync(h->w.counters + 1, 0, sizeof(int), h->st));
-  size_t sm = gat_smem(h);
+  CK(cudaMemsetAsync(h->w.counters + 2, 0, 2 * sizeof(int), h->st));
   {
     // algorithmic bytes: the acceleration mesh once, particles read and written
     Timed tm(h, KC_GATHER, 3.0 * real_bytes(h) + 64.0 * h->N);
     switch (h->r) {
 #define GATHER_R(R) \
-  case R: CK(launch_smem(parts::k_gather_push<R>, persistent_ctas(h), parts::GAT_NT, sm, h->st, &g)); break;
+  case R: CK(launch_smem(parts::k_gather_push<R>, persistent_ctas(h, parts::gat_ctas(R)), parts::gat_threads(R), parts::gat_smem_bytes<R>(), h->st, &g)); break;
       GATHER_R(2) GATHER_R(3) GATHER_R(4) GATHER_R(5) GATHER_R(6) GATHER_R(7)
 #undef GATHER_R
       default: return fail(h, MOND_EINVAL, "no gather for reach %d", h->r);
@@ -1241,21 +1237,12 @@ int mond_pm_create(mond_pm_grid grid, double box, double a0, double G, int mu_ki
           ball.push_back((uint32_t)(dx + h->r) | ((uint32_t)(dy + h->r) << 8) | ((uint32_t)(dz + h->r) << 16));
   h->nb = (int)ball.size();
   carve(n, h->r, h->nb, max_particles, (char*)workspace, &h->w);
-  // per-tap linear offsets: in the mesh (for balls away from the faces) and in
-  // a tile plus its reach (hw = 8 + 2r)
-  std::vector<int32_t> blin(h->nb), bhlin(h->nb);
   const int hw = parts::TILE + 2 * h->r;
-  for (int t = 0; t < h->nb; t++) {
-    int dx = ball[t] & 0xFF, dy = (ball[t] >> 8) & 0xFF, dz = (ball[t] >> 16) & 0xFF;
-    blin[t] = ((dz - h->r) * n + (dy - h->r)) * n + (dx - h->r);
-    bhlin[t] = (dz * hw + dy) * (hw + 1) + dx;  // tiles are staged with an odd x pitch hw + 1
-  }
   // rows (dy, dz) of the ball, each with its x extent L (dx in [-L, L]), for
-  // the row-wise deposit and gather: row k + 32 j goes to lane k. Two orders:
-  // the deposit's by decreasing L (lanes of a group have rows of similar
-  // length, so fewer predicated-off atomics); the gather's picks the 32 rows
-  // of each group with distinct tile offsets modulo 32 words where possible,
-  // so that the lanes' 16-byte loads at a given dx spread over the banks.
+  // the row-wise deposit and gather: by decreasing L, row k + 32 j goes to lane
+  // k of slot j. Inside a slot the rows are dealt so that each 16 lanes have
+  // distinct offsets modulo 16 cells where possible: their 8-byte loads at a
+  // given dx then take one pass over the banks.
   struct BallRow {
     int L, dy, dz, off;  // dy, dz shifted by r; off = tile offset of dx = 0
   };
@@ -1271,41 +1258,43 @@ int mond_pm_create(mond_pm_grid grid, double box, double a0, double G, int mu_ki
   const int nrows = (int)all.size();
   std::vector<BallRow> dep_order = all;
   std::stable_sort(dep_order.begin(), dep_order.end(), [](const BallRow& a, const BallRow& b) { return a.L > b.L; });
-  std::vector<std::vector<BallRow>> bucket(32);
-  for (const auto& b : all) bucket[b.off % 32].push_back(b);
-  std::vector<BallRow> gat_order;
-  while ((int)gat_order.size() < nrows) {
-    int taken = 0;  // one group: a row from each non-empty residue class in turn, then any
-    for (int b = 0; b < 32 && taken < 32; b++)
-      if (!bucket[b].empty()) {
-        gat_order.push_back(bucket[b].back());
-        bucket[b].pop_back();
-        taken++;
+  for (int k0 = 0; k0 < nrows; k0 += 32) {
+    const int k1 = std::min(nrows, k0 + 32);
+    std::vector<BallRow> left(dep_order.begin() + k0, dep_order.begin() + k1);
+    unsigned used = 0;
+    for (int k = k0; k < k1; k++) {
+      if ((k - k0) % 16 == 0) used = 0;
+      // among the rows whose residue is free, one of the most frequent residue left
+      int cnt[16] = {}, best = -1, score = -1;
+      for (const auto& b : left) cnt[b.off % 16]++;
+      for (int i = 0; i < (int)left.size(); i++) {
+        const int m = left[i].off % 16, sc = ((used >> m) & 1 ? 0 : 100) + cnt[m];
+        if (sc > score) score = sc, best = i;
       }
-    for (int b = 0; b < 32 && taken < 32; b++)
-      while (!bucket[b].empty() && taken < 32) {
-        gat_order.push_back(bucket[b].back());
-        bucket[b].pop_back();
-        taken++;
-      }
+      used |= 1u << (left[best].off % 16);
+      dep_order[k] = left[best];
+      left.erase(left.begin() + best);
+    }
   }
   h->nrows = nrows;
-  std::vector<int32_t> rowt(4 * nrows);  // deposit: [0, 2n), gather: [2n, 4n)
-  for (int k = 0; k < nrows; k++) {
-    rowt[k] = dep_order[k].off;
-    rowt[nrows + k] = dep_order[k].dy | (dep_order[k].dz << 8) | (dep_order[k].L << 16);
-    rowt[2 * nrows + k] = gat_order[k].off;
-    rowt[3 * nrows + k] = gat_order[k].dy | (gat_order[k].dz << 8) | (gat_order[k].L << 16);
-  }
+  std::vector<int32_t> rowt(nrows);
+  for (int k = 0; k < nrows; k++) rowt[k] = dep_order[k].dy | (dep_order[k].dz << 8) | (dep_order[k].L << 16);
   // per-axis lookup table of the Gaussian (Sect. 3.1): round(2^24 g1((j - r) - q/2^16))
-  const int lw = 2 * h->r + 1;
+  const int lw = parts::axis_pitch(h->r);  // rows padded to 16 bytes
   std::vector<uint32_t> lut((size_t)65537 * lw);
   for (int qi = 0; qi < 65537; qi++) {
     int q = qi - 32768;
-    for (int j = 0; j < lw; j++) {
+    for (int j = 0; j <= 2 * h->r; j++) {
       double u = (double)(j - h->r) - (double)q * (1.0 / 65536.0);
       lut[(size_t)qi * lw + j] = (uint32_t)nearbyint(g1(u, kernel_width) * 16777216.0);
     }
+  }
+  {
+    // the largest upper product word of the deposit's integer rule: the peak
+    // table word on every axis, the largest mass significand
+    const uint64_t w = (uint64_t)nearbyint(g1(0.0, kernel_width) * 16777216.0);
+    const uint64_t rmax = (w * w + 32768) >> 16, xmax = (w * 0xFFFFFFull + 32768) >> 16;
+    h->dep_max_sum = (uint32_t)(0xFFFFFFFFull / (((rmax * xmax) >> 32) + 1));
   }
   // twiddles (cos, sin)(2 pi m / n); wave numbers k and kappa = sin(k s)/s per index
   std::vector<float2> tw(n);
@@ -1338,8 +1327,6 @@ int mond_pm_create(mond_pm_grid grid, double box, double a0, double G, int mu_ki
   cudaError_t e = cudaSuccess;
   e = e ? e : cudaMemcpyAsync(h->w.lut, lut.data(), sizeof(uint32_t) * lut.size(), cudaMemcpyHostToDevice, h->st);
   e = e ? e : cudaMemcpyAsync(h->w.ball, ball.data(), sizeof(uint32_t) * ball.size(), cudaMemcpyHostToDevice, h->st);
-  e = e ? e : cudaMemcpyAsync(h->w.ball_lin, blin.data(), sizeof(int32_t) * h->nb, cudaMemcpyHostToDevice, h->st);
-  e = e ? e : cudaMemcpyAsync(h->w.ball_hlin, bhlin.data(), sizeof(int32_t) * h->nb, cudaMemcpyHostToDevice, h->st);
   e = e ? e : cudaMemcpyAsync(h->w.rows, rowt.data(), sizeof(int32_t) * rowt.size(), cudaMemcpyHostToDevice, h->st);
   e = e ? e : cudaMemcpyAsync(h->w.tw, tw.data(), sizeof(float2) * n, cudaMemcpyHostToDevice, h->st);
   e = e ? e : cudaMemcpyAsync(h->w.kv, kv.data(), sizeof(float) * n, cudaMemcpyHostToDevice, h->st);

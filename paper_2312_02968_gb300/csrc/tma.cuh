@@ -64,6 +64,10 @@ __device__ __forceinline__ void async_copy8_stream(void* dst, const void* src, u
                : "memory");
 }
 
+// Asynchronous 16-byte copy global -> shared (both 16-byte aligned; completes at async_wait_all).
+__device__ __forceinline__ void async_copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
 // Asynchronous 4-byte copy global -> shared (completes at async_wait_all).
 __device__ __forceinline__ void async_copy4(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
