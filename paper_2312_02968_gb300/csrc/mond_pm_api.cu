@@ -96,7 +96,7 @@ size_t carve(int n, int r, int nb, int64_t maxp, char* base, Workspace* w) {
     return p;
   };
   const int64_t n3 = (int64_t)n * n * n;
-  const int64_t plane = (int64_t)n * n * (n / 2 + 2);
+  const int64_t plane = (int64_t)n * n * passes::sp_of(n);
   const int ntx = n / parts::TILE;
   const int ntile = ntx * ntx * ntx;
   const int lw = parts::axis_pitch(r);
@@ -151,7 +151,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 bool encode_spectral_map(tma::TensorMap* m, void* base, int n, int ncomp, int bx, int by, int bz) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
-  const int sp = n / 2 + 2;
+  const int sp = passes::sp_of(n);
   cuuint64_t dims[3] = {(cuuint64_t)2 * sp, (cuuint64_t)n, (cuuint64_t)ncomp * n};
   cuuint64_t strides[2] = {(cuuint64_t)2 * sp * 4, (cuuint64_t)2 * sp * 4 * n};
   cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
@@ -167,7 +167,7 @@ bool encode_spectral_map(tma::TensorMap* m, void* base, int n, int ncomp, int bx
 bool encode_component_map(tma::TensorMap* m, void* base, int n, int ncomp, int bx, int bc, int bz, int cstep = 1) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
-  const int sp = n / 2 + 2;
+  const int sp = passes::sp_of(n);
   const cuuint64_t row = (cuuint64_t)2 * sp * 4, plane = row * n * n;
   cuuint64_t dims[4] = {(cuuint64_t)2 * sp, (cuuint64_t)ncomp, (cuuint64_t)n, (cuuint64_t)n};
   cuuint64_t strides[3] = {plane * cstep, row, row * n};
@@ -185,7 +185,7 @@ bool encode_component_map(tma::TensorMap* m, void* base, int n, int ncomp, int b
 bool encode_row_component_map(tma::TensorMap* m, void* base, int n, int ncomp, int bx, int by) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return false;
-  const int sp = n / 2 + 2;
+  const int sp = passes::sp_of(n);
   const cuuint64_t row = (cuuint64_t)2 * sp * 4, plane = row * n * n;
   cuuint64_t dims[4] = {(cuuint64_t)2 * sp, (cuuint64_t)ncomp, (cuuint64_t)n, (cuuint64_t)n};
   cuuint64_t strides[3] = {plane, row, row * n};
@@ -1220,7 +1220,7 @@ int mond_pm_create(mond_pm_grid grid, double box, double a0, double G, int mu_ki
   h->st = (cudaStream_t)cuda_stream;
   const int n = h->nf;
   h->n3 = (int64_t)n * n * n;
-  h->plane = (int64_t)n * n * (n / 2 + 2);
+  h->plane = (int64_t)n * n * passes::sp_of(n);
   h->ntx = n / parts::TILE;
   h->ntile = h->ntx * h->ntx * h->ntx;
   int dev = 0;

@@ -22,19 +22,27 @@ namespace passes {
 constexpr int NT = 256;   // threads per CTA of the y- and z-passes
 constexpr int NTX = 256;  // threads per CTA of the x-pass
 
+// Complex values of a spectral row in memory: N/2 + 1 rounded up so that every
+// row starts on a 32-byte sector, and so does every tile of four columns (rows
+// of N/2 + 2 begin in the middle of a sector every other time, and a tile row
+// of 32 or 64 bytes then moves a sector more): 512^3 curl-free z-step 1.15 ->
+// 0.88 ms, final 1.27 -> 0.88 ms, y-unfold 0.76 -> 0.59 ms; 256^3 y-passes 5%
+// and z-passes 3 to 8% less.
+constexpr int sp_of(int n) { return n / 2 + 4; }
+
 template <int N>
 struct XCfg {
   static constexpr int L = N >= 384 ? 8 : 16;  // lines per CTA
   static constexpr int LP = L + 1;             // padded line pitch in shared memory (bank spread)
   static constexpr int H = N / 2;              // complex FFT length of the real transform
   static constexpr int ROWS = H + 1;           // spectral positions 0..N/2
-  static constexpr int SP = N / 2 + 2;
+  static constexpr int SP = sp_of(N);
 };
 
 template <int N>
 struct YZCfg {
   static constexpr int P = N >= 384 ? 8 : 16;    // kx columns per tile
-  static constexpr int SP = N / 2 + 2;
+  static constexpr int SP = sp_of(N);
   static constexpr int NX = N / 2 + 1;           // valid kx columns
   static constexpr int NBLK = (NX + P - 1) / P;  // tiles across kx
 };
@@ -274,7 +282,7 @@ __device__ __forceinline__ void x_store_spec(const float2* sm, float2* __restric
   for (int l = warp; l < C::L; l += NTX / 32) {
     for (int qq = lane; qq < Q; qq += 32) {
       const int kk = 2 * qq;
-      float2 a = sm[kk * C::LP + l];
+      float2 a = (kk <= C::H) ? sm[kk * C::LP + l] : make_float2(0.f, 0.f);
       float2 b = (kk + 1 <= C::H) ? sm[(kk + 1) * C::LP + l] : make_float2(0.f, 0.f);
       __stcs(dst + l * Q + qq, make_float4(a.x, a.y, b.x, b.y));
     }
@@ -1188,7 +1196,7 @@ __global__ void __launch_bounds__(NTY, 3) k_ypass_fold(const __grid_constant__ t
   constexpr int H = N / 2;
   constexpr int NBF = (H + 1 + PF - 1) / PF;  // folded blocks; the last holds kx = N/2
   constexpr int NBP = (H + 1 + PP - 1) / PP;  // plain blocks
-  constexpr int SP = N / 2 + 2;
+  constexpr int SP = sp_of(N);
   constexpr int BOX = pipe_box(N), NBOX = N / BOX;
   constexpr int DIR = KIND == YF_FOLD ? -1 : +1;
   constexpr int R = N * PP;   // elements of a stage
