@@ -95,8 +95,8 @@ enum {
                              when an argument, option or binding changes; needs a non-default stream and
                              is bypassed while MOND_OPT_TIMING is on (default 0) */
   MOND_OPT_TIMING = 4,    /* value 1: bracket every launch with CUDA events (see mond_pm_kernel_stats) */
-  MOND_OPT_PIPELINED = 5, /* value 1 (default): y/z passes stream tiles with TMA through a two-stage ring;
-                             0: one tile per CTA with plain loads (same results) */
+  MOND_OPT_PIPELINED = 5, /* value 1 (default): y/z passes with their transforms in registers;
+                             0: in shared memory, with plain loads (same results up to FP32 rounding order) */
   MOND_OPT_CHUNK = 6,     /* particles per deposit/gather work item at most: a power of two in 256..4096
                              (default 1024; a small system's items are smaller; same results) */
   MOND_OPT_GATHER = 7,    /* force at the particles. 0 (default): Eq. gi, the ball sum at each particle.
@@ -120,14 +120,13 @@ enum {
                              the solution of the discretised equation); the mean is the cycle's midpoint.
                              Not in the paper. Costs one half-spectrum plane written and read. Needs
                              MOND_OPT_PIPELINED 1 (default 0) */
-  MOND_OPT_FOLD = 10,         /* value 1 (default): where the pipelined passes run and the side allows it
-                             (every supported side but 16 and 48), the curl-free, final and Newton steps
+  MOND_OPT_FOLD = 10,         /* value 1 (default): where MOND_OPT_PIPELINED is 1, the curl-free, final and Newton steps
                              carry one scalar and its z-derivative between their y- and z-passes instead
                              of three components (the gradient form of their operators, with the axes on a
                              Nyquist plane kept apart); 0: three components throughout. Same results up to
                              FP32 rounding order. */
-  MOND_OPT_GRID_CAP = 11      /* value c > 0: the persistent kernels of a step (pipelined y/z passes,
-                             deposit, gather) launch at most c CTAs, leaving the rest of the GPU to
+  MOND_OPT_GRID_CAP = 11      /* value c > 0: the y/z passes, the deposit and the gather of a step
+                             launch at most c CTAs (each working on several tiles), leaving the rest of the GPU to
                              kernels that run beside them (independent systems on their own streams,
                              a batch); 0 (default): as many as fit the GPU. Same results. */
 };

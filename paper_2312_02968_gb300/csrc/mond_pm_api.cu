@@ -162,41 +162,6 @@ bool encode_spectral_map(tma::TensorMap* m, void* base, int n, int ncomp, int bx
   return r == CUDA_SUCCESS;
 }
 
-// 4-D view (x: 2 SP floats, component: ncomp planes cstep planes apart, y: N
-// rows, z: N planes) with box (bx, bc, 1, bz): z-pass tiles [z][component][column].
-bool encode_component_map(tma::TensorMap* m, void* base, int n, int ncomp, int bx, int bc, int bz, int cstep = 1) {
-  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!enc) return false;
-  const int sp = passes::sp_of(n);
-  const cuuint64_t row = (cuuint64_t)2 * sp * 4, plane = row * n * n;
-  cuuint64_t dims[4] = {(cuuint64_t)2 * sp, (cuuint64_t)ncomp, (cuuint64_t)n, (cuuint64_t)n};
-  cuuint64_t strides[3] = {plane * cstep, row, row * n};
-  cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)bc, 1, (cuuint32_t)bz};
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  CUresult r = enc(reinterpret_cast<CUtensorMap*>(m), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box, es,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
-// 4-D view (x: 2 SP floats, component: ncomp planes, y: N rows, z: N planes)
-// with box (bx, 2, by, 1): folded y-pass tiles [row][component][column] of
-// components 0 and 1.
-bool encode_row_component_map(tma::TensorMap* m, void* base, int n, int ncomp, int bx, int by) {
-  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!enc) return false;
-  const int sp = passes::sp_of(n);
-  const cuuint64_t row = (cuuint64_t)2 * sp * 4, plane = row * n * n;
-  cuuint64_t dims[4] = {(cuuint64_t)2 * sp, (cuuint64_t)ncomp, (cuuint64_t)n, (cuuint64_t)n};
-  cuuint64_t strides[3] = {plane, row, row * n};
-  cuuint32_t box[4] = {(cuuint32_t)bx, 2, (cuuint32_t)by, 1};
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  CUresult r = enc(reinterpret_cast<CUtensorMap*>(m), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box, es,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
 // Gaussian of Eq. smooth along one axis, width sigma pixels.
 double g1(double u, double sigma) { return exp(-(u * u) / (2.0 * sigma * sigma)) / (sigma * sqrt(2.0 * M_PI)); }
 
@@ -357,13 +322,9 @@ struct mond_pm {
     }
   } gkey{};
   int64_t glaunches = 0;
-  // TMA views of the spectral buffers: y-pass tiles (3-D), z-pass tiles with
-  // the component as a dimension (4-D; W with 1 or 3 components per box, A
-  // with 3 or 4)
-  tma::TensorMap map_wy, map_ay, map_wz1, map_wz3, map_az1, map_az3;
-  // the folded passes: y tiles of two components (narrower), z tiles of components 0 and 2
-  tma::TensorMap map_wyf, map_ayf, map_wy4, map_ay4, map_wz02, map_az02;
-  bool fold_maps = false;
+  // TMA views of the spectral buffers for the staged y-pass of the bounded-wait tests
+  tma::TensorMap map_wy, map_ay;
+  bool maps = false;
   std::vector<TimedLaunch> tl;      // launches recorded since the last read
   std::vector<cudaEvent_t> evpool;  // recycled events
   int64_t st_launch[KC_COUNT] = {};
@@ -476,13 +437,48 @@ cudaError_t xpass(mond_pm* h, int mode, passes::XArgs a) {
   return cudaErrorInvalidValue;
 }
 
+cudaError_t yreg(mond_pm* h, int kind, const regpass::YRegArgs& p) {
+  switch (h->nf) {
+#define MOND_CASE(k) \
+  case k: return mond_yreg_##k(kind, p, h->grid_cap, h->st);
+    MOND_SIZES(MOND_CASE)
+#undef MOND_CASE
+  }
+  return cudaErrorInvalidValue;
+}
+
+// Register z-pass on the planes in -> out; the potential's slot is component 3 of A.
+cudaError_t zreg(mond_pm* h, int mode, bool fold, const float2* in, float2* out, int nout, int mean) {
+  regpass::ZRegArgs p{};
+  p.in = in;
+  p.out = out;
+  p.scal = h->w.A + 3 * h->plane;
+  p.pstride = h->plane;
+  p.mean = mean;
+  p.kv = h->w.kv;
+  p.kp = h->w.kp;
+  p.tw = h->w.tw;
+  // the final pass multiplies by the smoothing spectrum only for the interpolating gather
+  p.khat = (mode == passes::Z_SMOOTH || (mode == passes::Z_FINAL && h->gather_mode)) ? h->w.khat : nullptr;
+  p.norm = (float)(1.0 / ((double)h->nf * h->nf * h->nf));
+  p.coef = (float)(4.0 * M_PI * h->G);
+  switch (h->nf) {
+#define MOND_CASE(k) \
+  case k: return mond_zreg_##k(mode, fold, nout > 3, p, h->grid_cap, h->st);
+    MOND_SIZES(MOND_CASE)
+#undef MOND_CASE
+  }
+  return cudaErrorInvalidValue;
+}
+
 cudaError_t ypass(mond_pm* h, int dir, float2* spec, int ncomp) {
-  if (h->pipelined) {
+  if (h->pipelined && h->lost_tile >= 0) {
+    // fault injection of the bounded-wait tests (one-shot): the pass whose tiles are staged by TMA
     passes::PipeYArgs p{};
     p.ncomp = ncomp;
     p.tw = h->w.tw;
     p.status = h->w.status;
-    p.lost_tile = h->lost_tile;  // fault injection of the bounded-wait tests (one-shot)
+    p.lost_tile = h->lost_tile;
     p.max_ctas = h->grid_cap;
     h->lost_tile = -1;
     const tma::TensorMap& m = spec == h->w.W ? h->map_wy : h->map_ay;
@@ -494,6 +490,15 @@ cudaError_t ypass(mond_pm* h, int dir, float2* spec, int ncomp) {
 #undef MOND_CASE
     }
     return cudaErrorInvalidValue;
+  }
+  if (h->pipelined) {
+    regpass::YRegArgs p{};
+    p.spec = spec;
+    p.pstride = h->plane;
+    p.nplain = ncomp;
+    p.tw = h->w.tw;
+    Timed tm(h, dir < 0 ? KC_Y_FWD : KC_Y_INV, 2.0 * ncomp * spec_bytes(h));
+    return yreg(h, dir < 0 ? regpass::Y_FWD : regpass::Y_INV, p);
   }
   passes::YArgs a{};
   a.spec = spec;
@@ -529,31 +534,7 @@ cudaError_t zpass(mond_pm* h, int mode, float2* in, float2* out, int nout, int m
   int zc = mode == passes::Z_NEWTON ? KC_Z_NEWTON : mode == passes::Z_CURL ? KC_Z_CURL : mode == passes::Z_DIV ? KC_Z_DIV
            : mode == passes::Z_FINAL ? KC_Z_FINAL : KC_Z_SMOOTH;
   Timed tm(h, zc, zb);
-  if (h->pipelined) {
-    passes::PipeZArgs p{};
-    p.nout = nout;
-    p.kv = a.kv;
-    p.kp = a.kp;
-    p.tw = a.tw;
-    p.khat = a.khat;
-    p.norm = a.norm;
-    p.coef = a.coef;
-    p.status = h->w.status;
-    p.mean = mean;
-    p.max_ctas = h->grid_cap;
-    // input: rho^ (component 0 of W) for Newton, else three components;
-    // output: three components, phi^ separately as component 3 of A
-    const tma::TensorMap& mi =
-        in == h->w.W ? (mode == passes::Z_NEWTON ? h->map_wz1 : h->map_wz3) : h->map_az3;
-    const tma::TensorMap& mo = out == h->w.W ? h->map_wz3 : h->map_az3;
-    switch (h->nf) {
-#define MOND_CASE(k) \
-  case k: return mond_zpass_pipe_##k(mode, mi, mo, h->map_az1, p, h->st);
-      MOND_SIZES(MOND_CASE)
-#undef MOND_CASE
-    }
-    return cudaErrorInvalidValue;
-  }
+  if (h->pipelined) return zreg(h, mode, false, in, out, nwr, mean);
   if (mean) return cudaErrorInvalidValue;  // the mean of the last two iterations needs the pipelined passes
   switch (h->nf) {
 #define MOND_CASE(k) \
@@ -566,95 +547,36 @@ cudaError_t zpass(mond_pm* h, int mode, float2* in, float2* out, int nout, int m
 
 // Whether a solve takes the folded y/z passes around its curl-free, final and
 // Newton steps.
-bool use_fold(const mond_pm* h) { return h->fold && h->pipelined && h->fold_maps; }
+bool use_fold(const mond_pm* h) { return h->fold && h->pipelined; }
 
-// Folded y-pass (passes::YF_*): forward before a curl-free or final z-pass,
-// inverse after a folded z-pass; nplain components from 2 on are transformed
-// as they are.
+// Folded y-pass (regpass::Y_FOLD ..): forward before a curl-free or final
+// z-pass, inverse after a folded z-pass; nplain components from 2 on are
+// transformed as they are.
 cudaError_t yfold(mond_pm* h, int kind, float2* spec, int nplain) {
-  passes::PipeYFArgs p{};
-  p.nplain = nplain;
-  p.tw = h->w.tw;
-  p.kt = (kind == passes::YF_GRAD || kind == passes::YF_GRADN) ? h->w.kp : h->w.kv;
+  regpass::YRegArgs p{};
   p.spec = spec;
   p.pstride = h->plane;
-  p.status = h->w.status;
-  p.max_ctas = h->grid_cap;
-  const bool w = spec == h->w.W;
-  const double S = spec_bytes(h);
+  p.c0 = 2;
+  p.nplain = nplain;
+  p.tw = h->w.tw;
+  p.kt = (kind == regpass::Y_GRAD || kind == regpass::Y_GRADN) ? h->w.kp : h->w.kv;
   // the folded pair: two components in and one out (fold), or one in and two
-  // out (unfold; the kx = N/2 block of the curl-free kind reads two); plain
-  // components one in, one out
-  const double bytes = 3.0 * S + 2.0 * nplain * S;
-  Timed tm(h, kind == passes::YF_FOLD ? KC_Y_FOLD : KC_Y_UNFOLD, bytes);
-  switch (h->nf) {
-#define MOND_CASE(k) \
-  case k:                                                                                               \
-    return mond_ypass_fold_##k(kind, w ? h->map_wy4 : h->map_ay4, w ? h->map_wyf : h->map_ayf,           \
-                               w ? h->map_wy : h->map_ay, p, h->st);
-    MOND_SIZES(MOND_CASE)
-#undef MOND_CASE
-  }
-  return cudaErrorInvalidValue;
+  // out (unfold); plain components one in, one out
+  const double S = spec_bytes(h);
+  Timed tm(h, kind == regpass::Y_FOLD ? KC_Y_FOLD : KC_Y_UNFOLD, 3.0 * S + 2.0 * nplain * S);
+  return yreg(h, kind, p);
 }
 
 // Folded z-pass: Z_NEWTON (rho^ in component 0 of W), Z_CURL (in place on W)
-// or Z_FINAL (W to out). The tiles holding kx = N/2 or ky = N/2 of the last
-// two go through k_zpass_pipe first (three components, as unfolded), the
-// others through the folded kernel (components 0 and 2).
+// or Z_FINAL (W to out).
 cudaError_t zfold(mond_pm* h, int mode, float2* out, int nout, int mean = 0) {
-  passes::PipeZArgs p{};
-  p.nout = nout;
-  p.kv = h->w.kv;
-  p.kp = h->w.kp;
-  p.tw = h->w.tw;
-  p.khat = (mode == passes::Z_FINAL && h->gather_mode) ? h->w.khat : nullptr;
-  p.norm = (float)(1.0 / ((double)h->nf * h->nf * h->nf));
-  p.coef = (float)(4.0 * M_PI * h->G);
-  p.status = h->w.status;
-  p.mean = mean;
-  p.max_ctas = h->grid_cap;
-  const bool toA = out == h->w.A;
   const int zc = mode == passes::Z_NEWTON ? KC_Z_NEWTON : mode == passes::Z_CURL ? KC_Z_CURL : KC_Z_FINAL;
   const double S = spec_bytes(h);
-  const double extra = ((mode != passes::Z_CURL && nout > 3) ? S : 0.0) + (mean ? S : 0.0) +
-                       (p.khat ? 0.5 * real_bytes(h) : 0.0);  // potential out, kept potential, smoothing spectrum
-  if (mode != passes::Z_NEWTON) {
-    const int pz = passes::pipe_pz(h->nf);
-    const double nblk = (h->nf / 2 + pz) / pz, ffull = (nblk + h->nf - 1) / (nblk * h->nf);
-    p.nyq_only = 1;
-    {
-      Timed tm(h, zc, (6.0 * S + extra) * ffull);
-      switch (h->nf) {
-#define MOND_CASE(k) \
-  case k: {                                                                                                      \
-    cudaError_t e = mond_zpass_pipe_##k(mode, h->map_wz3, toA ? h->map_az3 : h->map_wz3, h->map_az1, p, h->st); \
-    if (e != cudaSuccess) return e;                                                                              \
-    break;                                                                                                       \
-  }
-        MOND_SIZES(MOND_CASE)
-#undef MOND_CASE
-        default: return cudaErrorInvalidValue;
-      }
-    }
-    p.nyq_only = 0;
-    Timed tm(h, zc, (4.0 * S + extra) * (1.0 - ffull));
-    switch (h->nf) {
-#define MOND_CASE(k) \
-  case k: return mond_zpass_fold_##k(mode, h->map_wz02, toA ? h->map_az02 : h->map_wz02, h->map_az1, p, h->st);
-      MOND_SIZES(MOND_CASE)
-#undef MOND_CASE
-    }
-    return cudaErrorInvalidValue;
-  }
-  Timed tm(h, zc, 3.0 * S + extra);
-  switch (h->nf) {
-#define MOND_CASE(k) \
-  case k: return mond_zpass_fold_##k(mode, h->map_wz1, toA ? h->map_az02 : h->map_wz02, h->map_az1, p, h->st);
-    MOND_SIZES(MOND_CASE)
-#undef MOND_CASE
-  }
-  return cudaErrorInvalidValue;
+  // two components in (Newton one) and two out; potential out, kept potential, smoothing spectrum
+  const double bytes = (mode == passes::Z_NEWTON ? 3.0 : 4.0) * S + ((mode != passes::Z_CURL && nout > 3) ? S : 0.0) +
+                       (mean ? S : 0.0) + (mode == passes::Z_FINAL && h->gather_mode ? 0.5 * real_bytes(h) : 0.0);
+  Timed tm(h, zc, bytes);
+  return zreg(h, mode, true, h->w.W, out, nout, mean);
 }
 
 #define PK(call)                                                                            \
@@ -929,7 +851,7 @@ int do_solve(mond_pm* h, int K, int warm, const float* Hguess) {
     if (K == 0) {
       if (fold) {
         PK(zfold(h, passes::Z_NEWTON, A, nout));
-        PK(yfold(h, passes::YF_GRAD, A, nout - 2));
+        PK(yfold(h, regpass::Y_GRAD, A, nout - 2));
       } else {
         PK(zpass(h, passes::Z_NEWTON, W, A, nout));
         PK(ypass(h, +1, A, nout));
@@ -953,7 +875,7 @@ int do_solve(mond_pm* h, int K, int warm, const float* Hguess) {
     }
     if (fold) {
       PK(zfold(h, passes::Z_NEWTON, W, 3));
-      PK(yfold(h, passes::YF_GRAD, W, 1));
+      PK(yfold(h, regpass::Y_GRAD, W, 1));
     } else {
       PK(zpass(h, passes::Z_NEWTON, W, W, 3));
       PK(ypass(h, +1, W, 3));
@@ -993,7 +915,7 @@ int do_solve(mond_pm* h, int K, int warm, const float* Hguess) {
   PK(xpass(h, reuse ? passes::X_NU_REAL : passes::X_NU_FIRST, xn));
   h->gn_valid = true;
   for (int j = 1; j <= K; j++) {
-    if (fold) PK(yfold(h, passes::YF_FOLD, W, 1));
+    if (fold) PK(yfold(h, regpass::Y_FOLD, W, 1));
     else PK(ypass(h, -1, W, 3));
     const bool last = (j == K);
     if (last) {
@@ -1003,7 +925,7 @@ int do_solve(mond_pm* h, int K, int warm, const float* Hguess) {
       }
       if (fold) {
         PK(zfold(h, passes::Z_FINAL, A, nout, mean2 ? 2 : 0));
-        PK(yfold(h, passes::YF_GRADN, A, nout - 2));
+        PK(yfold(h, regpass::Y_GRADN, A, nout - 2));
       } else {
         PK(zpass(h, passes::Z_FINAL, W, A, nout, mean2 ? 2 : 0));
         PK(ypass(h, +1, A, nout));
@@ -1020,7 +942,7 @@ int do_solve(mond_pm* h, int K, int warm, const float* Hguess) {
     // last keeps its potential in the scalar slot of A (unused until Z_FINAL)
     if (fold) {
       PK(zfold(h, passes::Z_CURL, W, 3, (mean2 && j == K - 1) ? 1 : 0));
-      PK(yfold(h, passes::YF_CURL, W, 1));
+      PK(yfold(h, regpass::Y_CURL, W, 1));
     } else {
       PK(zpass(h, passes::Z_CURL, W, W, 3, (mean2 && j == K - 1) ? 1 : 0));
       PK(ypass(h, +1, W, 3));
@@ -1308,21 +1230,9 @@ int mond_pm_create(mond_pm_grid grid, double box, double a0, double G, int mu_ki
     kp[m] = (2 * m == n) ? 0.0f : (float)(sin(2.0 * M_PI * f / n) / h->s);
   }
   {
-    const int py = passes::pipe_py(n), pz = passes::pipe_pz(n), bx = passes::pipe_box(n);
-    bool ok = encode_spectral_map(&h->map_wy, h->w.W, n, 3, 2 * py, bx, 1) &&
-              encode_spectral_map(&h->map_ay, h->w.A, n, 4, 2 * py, bx, 1) &&
-              encode_component_map(&h->map_wz1, h->w.W, n, 3, 2 * pz, 1, bx) &&
-              encode_component_map(&h->map_wz3, h->w.W, n, 3, 2 * pz, 3, bx) &&
-              encode_component_map(&h->map_az1, h->w.A, n, 4, 2 * pz, 1, bx) &&
-              encode_component_map(&h->map_az3, h->w.A, n, 4, 2 * pz, 3, bx);
-    if (!ok) h->pipelined = 0;  // no driver entry point: the unpipelined passes
-    const int pyf = passes::pipe_pyf(n);
-    h->fold_maps = ok && passes::fold_ok(n) && encode_spectral_map(&h->map_wyf, h->w.W, n, 3, 2 * pyf, bx, 1) &&
-                   encode_spectral_map(&h->map_ayf, h->w.A, n, 4, 2 * pyf, bx, 1) &&
-                   encode_row_component_map(&h->map_wy4, h->w.W, n, 3, 2 * pyf, bx) &&
-                   encode_row_component_map(&h->map_ay4, h->w.A, n, 4, 2 * pyf, bx) &&
-                   encode_component_map(&h->map_wz02, h->w.W, n, 2, 2 * pz, 2, bx, 2) &&
-                   encode_component_map(&h->map_az02, h->w.A, n, 2, 2 * pz, 2, bx, 2);
+    const int py = passes::pipe_py(n), bx = passes::pipe_box(n);
+    h->maps = encode_spectral_map(&h->map_wy, h->w.W, n, 3, 2 * py, bx, 1) &&
+              encode_spectral_map(&h->map_ay, h->w.A, n, 4, 2 * py, bx, 1);
   }
   cudaError_t e = cudaSuccess;
   e = e ? e : cudaMemcpyAsync(h->w.lut, lut.data(), sizeof(uint32_t) * lut.size(), cudaMemcpyHostToDevice, h->st);
@@ -1394,7 +1304,7 @@ int mond_pm_set_option(mond_pm_t h, int option, int64_t value) {
       return MOND_OK;
     case MOND_OPT_TEST_LOST_LOAD:
       if (value < 0 || value > (1 << 30)) return fail(h, MOND_EINVAL, "lost-load tile out of range");
-      if (value && (h->use_graph || !h->pipelined))
+      if (value && (h->use_graph || !h->pipelined || !h->maps))
         return fail(h, MOND_ESTATE, "the lost-load test needs MOND_OPT_PIPELINED 1 and MOND_OPT_USE_GRAPH 0");
       h->lost_tile = (int)value - 1;
       return MOND_OK;

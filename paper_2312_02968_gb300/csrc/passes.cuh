@@ -810,29 +810,27 @@ __global__ void __launch_bounds__(NT) k_zpass(ZArgs a) {
 }  // namespace passes
 
 // ===========================================================================
-// Pipelined y- and z-passes: persistent CTAs stream tiles through a two-stage
-// shared-memory ring. One thread issues TMA tile loads (completion on an
+// Staged y-pass (the bounded-wait tests; the passes of a solve are those of
+// regpass.cuh): persistent CTAs stream tiles through a two-stage shared-memory
+// ring. One thread issues TMA tile loads (completion on an
 // mbarrier) for tile i+1 and TMA stores of tile i-1 while all threads
 // transform tile i, so HBM traffic overlaps the shared-memory FFT.
 // ===========================================================================
 
 namespace passes {
 
-// Tile geometry of the pipelined passes: P columns per tile (y: PY, z: PZ),
+// Tile geometry: PY columns per tile,
 // row boxes of at most 256 (the TMA box limit) dividing N.
 constexpr int pipe_py(int n) { return n >= 384 ? 8 : 16; }
-constexpr int pipe_pz(int n) { return n >= 256 ? 4 : (n >= 192 ? 8 : 16); }
 constexpr int pipe_box(int n) { return n <= 256 ? n : (n % 256 == 0 ? 256 : 128); }
 
 template <int N>
 struct PipeCfg {
   static constexpr int PY = pipe_py(N);
-  static constexpr int PZ = pipe_pz(N);
   static constexpr int BOX = pipe_box(N);
   static constexpr int NBOX = N / BOX;
   static constexpr int NX = N / 2 + 1;
   static constexpr int NBLKY = (NX + PY - 1) / PY;
-  static constexpr int NBLKZ = (NX + PZ - 1) / PZ;
 };
 
 // Polls after which the wait for a tile whose load was never issued gives
@@ -847,25 +845,6 @@ struct PipeYArgs {
   // never issued, so its wait runs out (-1: none).
   int lost_tile = -1;
   int max_ctas = 0;  // cap on the persistent grid (0: as many as fit the GPU)
-};
-
-struct PipeZArgs {
-  int nout;  // Z_NEWTON / Z_FINAL outputs (3 or 4)
-  // mean of the last two iterations' potentials: 1 = this Z_CURL also writes
-  // its A k'.g (the potential's spectrum over i, before the inverse z
-  // transform) to the scalar slot of the final spectra; 2 = this Z_FINAL
-  // reads it back and takes the mean with its own. Needs the scalar region.
-  int mean;
-  // 1: only the tiles holding kx = N/2 or ky = N/2 (the rest is the folded z-pass's)
-  int nyq_only;
-  int max_ctas;  // cap on the persistent grid (0: as many as fit the GPU)
-  const float* kv;
-  const float* kp;
-  const float2* tw;
-  const float* khat;
-  float norm;
-  float coef;
-  uint32_t* status;
 };
 
 // Common ring driver. LoadF(tile, stage_ptr, bar) issues the loads of a tile
@@ -951,509 +930,6 @@ __global__ void __launch_bounds__(NT) k_ypass_pipe(const __grid_constant__ tma::
     for (int b = 0; b < C::NBOX; b++) tma::store_3d(&map, x, b * C::BOX, zz, src + b * C::BOX * P);
   };
   pipe_run(ntiles, stage0, SE, bars, a.status, load, compute, store, a.lost_tile);
-}
-
-// z-pass over the tile of (column block, y): forward z, the spectral
-// operator, inverse z. Each stage holds a vector region [z row][3][column]
-// (4-D maps with the component as a dimension, so one FFT call transforms the
-// three components) and, for Z_NEWTON and Z_FINAL, a scalar region
-// [z row][column] for rho^ (input) or phi^ (output, component 3 of A).
-// threads per pipelined z-pass CTA: at N = 256, 192 = one radix-16 butterfly
-// per thread for the 3 x 4 sequences of a tile (four CTAs per SM); 384 elsewhere.
-template <int N, int MODE>
-constexpr int zthreads() { return N == 256 ? 192 : 384; }
-
-// SC: a separate scalar region per stage (needed only when phi is stored);
-// without it the Newton pass lands its scalar input in the last third of the
-// vector region and reads it into registers before the outputs overwrite it,
-// so that every mode runs with three-component stages (two CTAs per SM).
-template <int N, int MODE, bool SC, int NTZ = zthreads<N, MODE>()>
-__global__ void __launch_bounds__(NTZ, 768 / NTZ) k_zpass_pipe(const __grid_constant__ tma::TensorMap in_map,
-                                                   const __grid_constant__ tma::TensorMap out_map,
-                                                   const __grid_constant__ tma::TensorMap phi_map, PipeZArgs a) {
-  using C = PipeCfg<N>;
-  constexpr int P = C::PZ;
-  constexpr bool SCALAR = (MODE == Z_NEWTON || MODE == Z_FINAL);
-  constexpr int VP = 3 * P;                     // vector row pitch
-  constexpr int SE = N * VP + (SC ? N * P : 0);
-  constexpr int SOFF = SC ? N * VP : 2 * N * P;  // scalar region inside a stage
-  extern __shared__ __align__(128) float2 psm[];
-  __shared__ __align__(8) uint64_t bars[2];
-  float2* tw = psm;
-  float* kv = reinterpret_cast<float*>(psm + N);
-  float* kp = kv + N;
-  float2* stage0 = psm + 2 * N;
-  const bool phi = SC && SCALAR && a.nout > 3;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < N; i += NTZ) {
-    tw[i] = a.tw[i];
-    kv[i] = a.kv[i];
-    kp[i] = a.kp[i];
-  }
-  const int ntiles = a.nyq_only ? C::NBLKZ + N - 1 : C::NBLKZ * N;
-  // nyq_only: the row ky = N/2 of every block, then the block of kx = N/2 at every other row
-  auto tile_at = [&](int t, int& blk, int& y) {
-    if (!a.nyq_only) {
-      blk = t % C::NBLKZ;
-      y = t / C::NBLKZ;
-    } else if (t < C::NBLKZ) {
-      blk = t;
-      y = N / 2;
-    } else {
-      blk = C::NBLKZ - 1;
-      y = t - C::NBLKZ;
-      if (y >= N / 2) y++;
-    }
-  };
-  const bool mean_in = SC && MODE == Z_FINAL && a.mean == 2;   // previous potential read back
-  const bool mean_out = SC && MODE == Z_CURL && a.mean == 1;   // this iteration's potential kept
-  auto load = [&](int t, float2* dst, uint64_t* bar) -> uint32_t {
-    int blk, y;
-    tile_at(t, blk, y);
-    if constexpr (MODE == Z_NEWTON) {
-      tma::mbar_expect_tx(bar, N * P * 8);
-      for (int b = 0; b < C::NBOX; b++)
-        tma::load_4d(dst + SOFF + b * C::BOX * P, &in_map, blk * 2 * P, 0, y, b * C::BOX, bar);
-      return N * P * 8;
-    } else {
-      const uint32_t bytes = (mean_in ? 4 : 3) * N * P * 8;
-      tma::mbar_expect_tx(bar, bytes);
-      for (int b = 0; b < C::NBOX; b++) tma::load_4d(dst + b * C::BOX * VP, &in_map, blk * 2 * P, 0, y, b * C::BOX, bar);
-      if (mean_in)
-        for (int b = 0; b < C::NBOX; b++)
-          tma::load_4d(dst + SOFF + b * C::BOX * P, &phi_map, blk * 2 * P, 3, y, b * C::BOX, bar);
-      return bytes;
-    }
-  };
-  auto compute = [&](int t, float2* st) {
-    int blk, y;
-    tile_at(t, blk, y);
-    float2* sv = st;            // vector region
-    float2* ss = st + SOFF;     // scalar region
-    if constexpr (MODE == Z_NEWTON) fftk::fft<N, -1, P, NTZ>(ss, P, 1, tw, 1, tid);
-    else fftk::fft<N, -1, 3 * P, NTZ>(sv, VP, 1, tw, 1, tid);
-    const float ky = kv[y], kpy = kp[y];
-    const bool ny = (y == N / 2);
-    constexpr int PPT = (N * P + NTZ - 1) / NTZ;
-    float2 rin[(MODE == Z_NEWTON && !SC) ? PPT : 1];
-    if constexpr (MODE == Z_NEWTON && !SC) {
-      // the scalar input shares its space with the outputs: read it all first
-#pragma unroll
-      for (int k = 0; k < PPT; k++) {
-        const int i = tid + k * NTZ;
-        if (i < N * P) rin[k] = ss[i];
-      }
-      __syncthreads();
-    }
-#pragma unroll
-    for (int k = 0; k < PPT; k++) {
-      const int i = tid + k * NTZ;
-      if (i >= N * P) break;
-      const int row = i / P, cc = i % P, col = blk * P + cc;
-      if (col > N / 2) continue;
-      float2* v = sv + row * VP + cc;  // component c at v[c * P]
-      float2* sc = ss + row * P + cc;
-      const float kx = kv[col], kz = kv[row];
-      const bool nx = (col == N / 2), nz = (row == N / 2);
-      const float kk = kx * kx + ky * ky + kz * kz;
-      const float A = kk > 0.f ? __frcp_rn(kk) : 0.f;  // correctly rounded, as 1.0f / kk
-      if constexpr (MODE == Z_NEWTON) {
-        float2 r;
-        if constexpr (SC) r = *sc;
-        else r = rin[k];
-        const float f = a.coef * A * a.norm;  // 4 pi G A / N^3
-        const float2 ir = cmul_i<1>(r);
-        v[0] = cscale(ir, f * kp[col]);
-        v[P] = cscale(ir, f * kpy);
-        v[2 * P] = cscale(ir, f * kp[row]);
-        if constexpr (SC) *sc = cscale(r, -f);  // phi_N^ = -4 pi G A rho^
-      } else if constexpr (MODE == Z_SMOOTH) {
-        const float f = a.khat[((int64_t)row * N + y) * (N / 2 + 1) + col] * a.norm;
-        for (int c = 0; c < 3; c++) v[c * P] = cscale(v[c * P], f);
-      } else {
-        const float2 gg[3] = {v[0], v[P], v[2 * P]};
-        const float k3[3] = {kx, ky, kz};
-        const bool n3[3] = {nx, ny, nz};
-        if constexpr (MODE == Z_FINAL) {
-          // phi^ = i A sum_b k'_b g_b (k'_b = 0 on b's Nyquist plane); a^ = -i kappa phi^
-          float2 S = make_float2(0.f, 0.f);
-          for (int b = 0; b < 3; b++)
-            if (!n3[b]) S = cadd(S, cscale(gg[b], k3[b]));
-          float2 aS = cscale(S, A * a.norm);
-          if (mean_in) aS = cscale(cadd(aS, *sc), 0.5f);  // the midpoint of the last two iterations
-          // times the smoothing spectrum when the mesh is to hold the node-smoothed field
-          const float fk = a.khat ? a.khat[((int64_t)row * N + y) * (N / 2 + 1) + col] : 1.0f;
-          const float2 aK = cscale(aS, fk);
-          v[0] = cscale(aK, kp[col]);
-          v[P] = cscale(aK, kpy);
-          v[2 * P] = cscale(aK, kp[row]);
-          if constexpr (SC) *sc = cmul_i<1>(aS);
-        } else if (!(nx || ny || nz)) {
-          // away from the Nyquist planes (all but a few per cent of the points):
-          // P g = k (k.g) A, from one dot product
-          const float2 S = cadd(cadd(cscale(gg[0], kx), cscale(gg[1], ky)), cscale(gg[2], kz));
-          const float2 SA = cscale(S, A);
-          if (mean_out) *sc = cscale(SA, a.norm);  // the potential this step implies, as Z_FINAL forms it
-#pragma unroll
-          for (int aa = 0; aa < 3; aa++) {
-            const float2 acc = cscale(SA, k3[aa]);
-            v[aa * P] = cscale((MODE == Z_DIV) ? csub(gg[aa], acc) : acc, a.norm);
-          }
-        } else {
-          if (mean_out) {
-            // the potential this curl-free step implies, as Z_FINAL forms it: A sum_b k'_b g_b
-            float2 S = make_float2(0.f, 0.f);
-            for (int b = 0; b < 3; b++)
-              if (!n3[b]) S = cadd(S, cscale(gg[b], k3[b]));
-            *sc = cscale(S, A * a.norm);
-          }
-          // P_ab = k_a k_b A, off-diagonal terms dropped when exactly one of a, b is on its Nyquist plane
-          for (int aa = 0; aa < 3; aa++) {
-            float2 acc = make_float2(0.f, 0.f);
-            for (int b = 0; b < 3; b++)
-              if (aa == b || n3[aa] == n3[b]) acc = cadd(acc, cscale(gg[b], k3[aa] * k3[b] * A));
-            v[aa * P] = cscale((MODE == Z_DIV) ? csub(gg[aa], acc) : acc, a.norm);
-          }
-        }
-      }
-    }
-    __syncthreads();
-    fftk::fft<N, +1, 3 * P, NTZ>(sv, VP, 1, tw, 1, tid);
-    if (phi) fftk::fft<N, +1, P, NTZ>(ss, P, 1, tw, 1, tid);
-  };
-  auto store = [&](int t, const float2* src) {
-    int blk, y;
-    tile_at(t, blk, y);
-    const tma::TensorMap* m = SCALAR ? &out_map : &in_map;
-    for (int b = 0; b < C::NBOX; b++) tma::store_4d(m, blk * 2 * P, 0, y, b * C::BOX, src + b * C::BOX * VP);
-    if (phi || mean_out)
-      for (int b = 0; b < C::NBOX; b++)
-        tma::store_4d(&phi_map, blk * 2 * P, 3, y, b * C::BOX, src + N * VP + b * C::BOX * P);
-  };
-  pipe_run(ntiles, stage0, SE, bars, a.status, load, compute, store);
-}
-
-// ---------------------------------------------------------------------------
-// Folded passes around the curl-free, final and Newton z-passes.
-//
-// Away from the Nyquist planes the curl-free projection is the gradient of one
-// scalar, k (k.g) A, and the final and Newton operators are gradients too
-// (-i kappa phi^). So the y-pass before such a z-pass folds the x and y
-// components into s = kx gx^ + ky gy^ (component 0; component 2 keeps gz^),
-// the z-pass reads two components instead of three and writes the scalar u
-// and its z-derivative (components 0 and 2), and the y-pass after it unfolds
-// them into the three components again: kx u and ky u before its inverse
-// transform, the z one as it is.
-//
-// Where the Nyquist rule of the projection splits the axes into two sets (a
-// point on the kx = N/2 column or the ky = N/2 row) nothing is folded: the
-// fold stores gx^ and gy^ apart (the whole y-block holding kx = N/2; for the
-// other blocks the row ky = N/2, gy^ written to component 1 of that row
-// alone), k_zpass_pipe transforms the z-tiles holding kx = N/2 or ky = N/2
-// as it always does (nyq_only), and the unfold takes those values as they
-// are. The Newton step has no Nyquist rule (kappa vanishes there), so all its
-// tiles are folded. The z-block and the y-block holding kx = N/2 start at the
-// same column (fold_ok) so that the passes agree on which columns are apart.
-// ---------------------------------------------------------------------------
-// kx columns per folded tile of the folded y-passes: two components of
-// pyf columns, as many values as a plain tile of pipe_py(n) = 2 pyf columns
-constexpr int pipe_pyf(int n) { return pipe_py(n) / 2; }
-constexpr int yf_threads(int) { return NT; }
-
-constexpr bool fold_ok(int n) {
-  return n >= 32 && ((n / 2) / pipe_pyf(n)) * pipe_pyf(n) == ((n / 2) / pipe_pz(n)) * pipe_pz(n);
-}
-
-enum YFoldKind {
-  YF_FOLD = 0,   // forward: s = kx gx^ + ky gy^ into component 0
-  YF_CURL = 1,   // inverse after the curl-free z-pass: k_x u, k_y u (spectral k)
-  YF_GRADN = 2,  // inverse after the final z-pass: kappa_x u, kappa_y u
-  YF_GRAD = 3    // inverse after the Newton z-pass: as YF_GRADN, every row and block folded
-};
-
-struct PipeYFArgs {
-  int nplain;        // components transformed as they are: 2 .. 1 + nplain
-  const float2* tw;
-  const float* kt;   // per index: k (fold, curl) or kappa (gradients)
-  float2* spec;      // the spectral planes (component 1's row ky = N/2: plain loads and stores)
-  int64_t pstride;   // complex elements between components
-  uint32_t* status;
-  int max_ctas;      // cap on the persistent grid (0: as many as fit the GPU)
-};
-
-// Tiles of N x PP complex values (PP = pipe_py(N) = 2 pyf, 32 KB at N = 256,
-// the plain y-pass's tile): a plain tile holds PP columns of one component;
-// a folded tile holds pyf columns of components 0 and 1 interleaved per row,
-// [row][component][pyf], loaded and stored through a 4-D view with the
-// component as a dimension, so that all tiles take the same conflict-free
-// transform. The folded value s (fold) or u (unfold) travels as a compact
-// [row][pyf] block of component 0, packed and unpacked in place in two halves.
-template <int N, int KIND, int NTY = yf_threads(N)>
-__global__ void __launch_bounds__(NTY, 3) k_ypass_fold(const __grid_constant__ tma::TensorMap map4,
-                                                    const __grid_constant__ tma::TensorMap mapc,
-                                                    const __grid_constant__ tma::TensorMap mapp, PipeYFArgs a) {
-  constexpr int PF = pipe_pyf(N), PP = 2 * PF;
-  constexpr int H = N / 2;
-  constexpr int NBF = (H + 1 + PF - 1) / PF;  // folded blocks; the last holds kx = N/2
-  constexpr int NBP = (H + 1 + PP - 1) / PP;  // plain blocks
-  constexpr int SP = sp_of(N);
-  constexpr int BOX = pipe_box(N), NBOX = N / BOX;
-  constexpr int DIR = KIND == YF_FOLD ? -1 : +1;
-  constexpr int R = N * PP;   // elements of a stage
-  constexpr int RC = N * PF;  // elements of a compact block
-  constexpr int PER = R / 2 / NTY;  // slots per thread in each half of the tile
-  static_assert(R % (2 * NTY) == 0 && NTY % PP == 0 && PP <= 32, "slots split evenly, a warp on whole rows");
-  extern __shared__ __align__(128) float2 psm[];
-  __shared__ __align__(8) uint64_t bars[2];
-  float2* tw = psm;
-  float* kt = reinterpret_cast<float*>(psm + N);
-  float2* stage0 = psm + 2 * N;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < N; i += NTY) {
-    tw[i] = a.tw[i];
-    kt[i] = a.kt[i];
-  }
-  const int nxy = NBF * N;
-  const int ntiles = nxy + NBP * N * a.nplain;
-  // tile -> block, z and component (-1: the folded pair)
-  auto decode = [&](int t, int& blk, int& z, int& comp) {
-    if (t < nxy) {
-      blk = t % NBF;
-      z = t / NBF;
-      comp = -1;
-    } else {
-      const int u = t - nxy, rest = u / NBP;
-      blk = u % NBP;
-      comp = 2 + rest / N;
-      z = rest % N;
-    }
-  };
-  // whether a folded tile moves both components whole (else the compact block)
-  auto whole = [&](int blk) { return KIND == YF_FOLD ? false : (KIND != YF_GRAD && blk == NBF - 1); };
-  auto load = [&](int t, float2* dst, uint64_t* bar) -> uint32_t {
-    int blk, z, comp;
-    decode(t, blk, z, comp);
-    if (comp >= 0) {
-      tma::mbar_expect_tx(bar, R * 8);
-      for (int b = 0; b < NBOX; b++) tma::load_3d(dst + b * BOX * PP, &mapp, blk * 2 * PP, b * BOX, comp * N + z, bar);
-      return R * 8;
-    }
-    if (KIND == YF_FOLD || whole(blk)) {
-      tma::mbar_expect_tx(bar, R * 8);
-      for (int b = 0; b < NBOX; b++) tma::load_4d(dst + b * BOX * PP, &map4, blk * 2 * PF, 0, b * BOX, z, bar);
-      return R * 8;
-    }
-    tma::mbar_expect_tx(bar, RC * 8);
-    for (int b = 0; b < NBOX; b++) tma::load_3d(dst + b * BOX * PF, &mapc, blk * 2 * PF, b * BOX, z, bar);
-    return RC * 8;
-  };
-  auto compute = [&](int t, float2* st) {
-    int blk, z, comp;
-    decode(t, blk, z, comp);
-    float2* row1 = a.spec + a.pstride + ((int64_t)z * N + H) * SP;  // component 1, row ky = N/2
-    // per-element steps over the slots of the tile, a warp on two whole rows
-    // (lane q of a row: component q / PF, column q % PF)
-    const int q = tid % PP, c = q % PF;
-    const bool xs = q < PF;  // the x component's slot
-    const float kxc = kt[blk * PF + c];
-    if (comp < 0 && KIND != YF_FOLD && !whole(blk)) {
-      // unpack u: rows N/2.. first (their slots lie above every packed value),
-      // then rows ..N/2 - 1 (read all, then write)
-#pragma unroll
-      for (int half = 1; half >= 0; half--) {
-        float2 u[PER];
-#pragma unroll
-        for (int k = 0; k < PER; k++) {
-          const int row = (half * (R / 2) + tid + k * NTY) / PP;
-          u[k] = st[row * PF + c];
-        }
-        if (half == 0) __syncthreads();
-#pragma unroll
-        for (int k = 0; k < PER; k++) {
-          const int j = half * (R / 2) + tid + k * NTY, row = j / PP;
-          if (KIND != YF_GRAD && row == H)  // the Nyquist row: both outputs as the z-pass left them
-            st[j] = xs ? u[k] : row1[blk * PF + c];
-          else
-            st[j] = cscale(u[k], xs ? kxc : kt[row]);
-        }
-      }
-      __syncthreads();
-    }
-    fftk::fft<N, DIR, PP, NTY>(st, PP, 1, tw, 1, tid);
-    if (comp < 0 && KIND == YF_FOLD && blk != NBF - 1) {
-      // s = kx gx^ + ky gy^, packed: rows ..N/2 - 1 first (their packed places
-      // lie below every unread slot of the second half), then the rest; the
-      // y value reaches the x slot's lane by a shuffle
-#pragma unroll
-      for (int half = 0; half < 2; half++) {
-        float2 v[PER];
-#pragma unroll
-        for (int k = 0; k < PER; k++) {
-          const int j = half * (R / 2) + tid + k * NTY, row = j / PP;
-          const float2 mine = st[j];
-          const float2 other = make_float2(__shfl_xor_sync(0xffffffffu, mine.x, PF),
-                                           __shfl_xor_sync(0xffffffffu, mine.y, PF));
-          if (row == H) {
-            if (!xs) row1[blk * PF + c] = mine;  // gy^ of the Nyquist row, kept apart
-            v[k] = mine;
-          } else {
-            v[k] = cadd(cscale(mine, kxc), cscale(other, kt[row]));
-          }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < PER; k++) {
-          const int row = (half * (R / 2) + tid + k * NTY) / PP;
-          if (xs) st[row * PF + c] = v[k];
-        }
-      }
-    }
-  };
-  auto store = [&](int t, const float2* src) {
-    int blk, z, comp;
-    decode(t, blk, z, comp);
-    if (comp >= 0) {
-      for (int b = 0; b < NBOX; b++) tma::store_3d(&mapp, blk * 2 * PP, b * BOX, comp * N + z, src + b * BOX * PP);
-    } else if (KIND == YF_FOLD && blk != NBF - 1) {
-      for (int b = 0; b < NBOX; b++) tma::store_3d(&mapc, blk * 2 * PF, b * BOX, z, src + b * BOX * PF);
-    } else {
-      for (int b = 0; b < NBOX; b++) tma::store_4d(&map4, blk * 2 * PF, 0, b * BOX, z, src + b * BOX * PP);
-    }
-  };
-  pipe_run(ntiles, stage0, R, bars, a.status, load, compute, store);
-}
-
-// Folded z-pass (MODE Z_NEWTON, Z_CURL or Z_FINAL) over the tiles away from
-// the Nyquist planes of x and y (all tiles for Newton): it reads the folded
-// pair (s, gz^) through a map of components 0 and 2 ([z row][2][column] in
-// shared memory) and writes (u, z output) the same way; Newton reads rho^
-// (component 0) into the upper half of that region and takes it into
-// registers before its outputs overwrite it. The arithmetic per point is that of
-// k_zpass_pipe, with the x and y factors (k, or kappa for the gradients) left
-// to the unfolding y-pass. SCK: 1 = a scalar region for the mean of the last
-// two iterations, 2 = also the potential (its inverse z transform).
-template <int N, int MODE, int SCK>
-__global__ void __launch_bounds__(128, 6) k_zpass_fold(const __grid_constant__ tma::TensorMap in2,
-                                                       const __grid_constant__ tma::TensorMap out2,
-                                                       const __grid_constant__ tma::TensorMap phi_map, PipeZArgs a) {
-  constexpr int NTZ = 128;
-  using C = PipeCfg<N>;
-  constexpr int P = C::PZ;
-  constexpr int H = N / 2;
-  constexpr int R = N * P;
-  constexpr int IOFF = R;       // Newton: rho^, in the upper half of the pair's region (read out first)
-  constexpr int SOFF = 2 * R;   // scalar region
-  constexpr int SE = SOFF + (SCK ? R : 0);
-  constexpr int NBR = MODE == Z_NEWTON ? C::NBLKZ : C::NBLKZ - 1;  // column blocks visited
-  extern __shared__ __align__(128) float2 psm[];
-  __shared__ __align__(8) uint64_t bars[2];
-  float2* tw = psm;
-  float* kv = reinterpret_cast<float*>(psm + N);
-  float* kp = kv + N;
-  float2* stage0 = psm + 2 * N;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < N; i += NTZ) {
-    tw[i] = a.tw[i];
-    kv[i] = a.kv[i];
-    kp[i] = a.kp[i];
-  }
-  const int ntiles = MODE == Z_NEWTON ? NBR * N : NBR * (N - 1);
-  auto tile_at = [&](int t, int& blk, int& y) {
-    blk = t % NBR;
-    y = t / NBR;
-    if (MODE != Z_NEWTON && y >= H) y++;  // the row ky = N/2 is k_zpass_pipe's
-  };
-  const bool mean_in = SCK && MODE == Z_FINAL && a.mean == 2;
-  const bool mean_out = SCK && MODE == Z_CURL && a.mean == 1;
-  auto load = [&](int t, float2* dst, uint64_t* bar) -> uint32_t {
-    int blk, y;
-    tile_at(t, blk, y);
-    const uint32_t bytes = ((MODE == Z_NEWTON ? 1 : 2) + (mean_in ? 1 : 0)) * R * 8;
-    tma::mbar_expect_tx(bar, bytes);
-    for (int b = 0; b < C::NBOX; b++)
-      tma::load_4d(dst + (MODE == Z_NEWTON ? IOFF + b * C::BOX * P : b * C::BOX * 2 * P), &in2, blk * 2 * P, 0, y,
-                   b * C::BOX, bar);
-    if (mean_in)
-      for (int b = 0; b < C::NBOX; b++)
-        tma::load_4d(dst + SOFF + b * C::BOX * P, &phi_map, blk * 2 * P, 3, y, b * C::BOX, bar);
-    return bytes;
-  };
-  auto compute = [&](int t, float2* st) {
-    int blk, y;
-    tile_at(t, blk, y);
-    float2* ss = st + SOFF;
-    const float ky = kv[y];
-    constexpr int PPT = (R + NTZ - 1) / NTZ;
-    float2 rin[MODE == Z_NEWTON ? PPT : 1];
-    if constexpr (MODE == Z_NEWTON) {
-      fftk::fft<N, -1, P, NTZ>(st + IOFF, P, 1, tw, 1, tid);
-      // the outputs overwrite the input: take it all into registers first
-#pragma unroll
-      for (int k = 0; k < PPT; k++) {
-        const int i = tid + k * NTZ;
-        if (i < R) rin[k] = st[IOFF + i];
-      }
-      __syncthreads();
-    } else {
-      fftk::fft<N, -1, 2 * P, NTZ, 1>(st, 2 * P, 1, tw, 1, tid);
-    }
-#pragma unroll
-    for (int k = 0; k < PPT; k++) {
-      const int i = tid + k * NTZ;
-      if (i >= R) break;
-      const int row = i / P, cc = i % P, col = blk * P + cc;
-      if (col > H) continue;
-      const float kx = kv[col], kz = kv[row];
-      const float kk = kx * kx + ky * ky + kz * kz;
-      const float A = kk > 0.f ? __frcp_rn(kk) : 0.f;  // correctly rounded, as 1.0f / kk
-      float2* v = st + row * 2 * P + cc;  // u (in: s) at v[0], z output (in: gz^) at v[P]
-      if constexpr (MODE == Z_NEWTON) {
-        const float2 r = rin[k];
-        const float f = a.coef * A * a.norm;  // 4 pi G A / N^3
-        const float2 ir = cmul_i<1>(r);
-        v[0] = cscale(ir, f);
-        v[P] = cscale(ir, f * kp[row]);
-        if constexpr (SCK) ss[i] = cscale(r, -f);  // phi_N^ = -4 pi G A rho^
-      } else {
-        const bool nz = (row == H);
-        const float2 s = v[0], gz = v[P];
-        if constexpr (MODE == Z_CURL) {
-          if (!nz) {
-            const float2 SA = cscale(cadd(s, cscale(gz, kz)), A);
-            if (mean_out) ss[i] = cscale(SA, a.norm);
-            v[0] = cscale(SA, a.norm);
-            v[P] = cscale(cscale(SA, kz), a.norm);
-          } else {
-            // kz on its Nyquist plane: z is a set of its own
-            if (mean_out) ss[i] = cscale(s, A * a.norm);
-            v[0] = cscale(cscale(s, A), a.norm);
-            v[P] = cscale(cscale(gz, kz * kz * A), a.norm);
-          }
-        } else {  // Z_FINAL: phi^ = i A sum_b k'_b g_b (k'_z = 0 on its Nyquist plane), a^ = -i kappa phi^
-          const float2 S = nz ? s : cadd(s, cscale(gz, kz));
-          float2 aS = cscale(S, A * a.norm);
-          if (mean_in) aS = cscale(cadd(aS, ss[i]), 0.5f);  // the midpoint of the last two iterations
-          const float fk = a.khat ? a.khat[((int64_t)row * N + y) * (N / 2 + 1) + col] : 1.0f;
-          const float2 aK = cscale(aS, fk);
-          v[0] = aK;
-          v[P] = cscale(aK, kp[row]);
-          if constexpr (SCK == 2) ss[i] = cmul_i<1>(aS);
-        }
-      }
-    }
-    __syncthreads();
-    fftk::fft<N, +1, 2 * P, NTZ, 1>(st, 2 * P, 1, tw, 1, tid);
-    if constexpr (SCK == 2) fftk::fft<N, +1, P, NTZ>(ss, P, 1, tw, 1, tid);
-  };
-  auto store = [&](int t, const float2* src) {
-    int blk, y;
-    tile_at(t, blk, y);
-    for (int b = 0; b < C::NBOX; b++) tma::store_4d(&out2, blk * 2 * P, 0, y, b * C::BOX, src + b * C::BOX * 2 * P);
-    if (SCK == 2 || mean_out)
-      for (int b = 0; b < C::NBOX; b++)
-        tma::store_4d(&phi_map, blk * 2 * P, 3, y, b * C::BOX, src + SOFF + b * C::BOX * P);
-  };
-  pipe_run(ntiles, stage0, SE, bars, a.status, load, compute, store);
 }
 
 }  // namespace passes

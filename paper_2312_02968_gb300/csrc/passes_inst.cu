@@ -1,7 +1,7 @@
 // passes_inst.cu -- host launchers of the mesh passes for one FFT-domain side
 // N = MOND_N (this file is compiled once per supported size, in parallel).
-#include "passes.cuh"
 #include "launch.h"
+#include "regpass.cuh"
 
 #ifndef MOND_N
 #error "compile with -DMOND_N=<size>"
@@ -105,31 +105,6 @@ cudaError_t launch_ypipe(const tma::TensorMap& map, const PipeYArgs& a, cudaStre
   return cudaGetLastError();
 }
 
-template <int MODE, bool SC>
-cudaError_t launch_zpipe_sc(const tma::TensorMap& in, const tma::TensorMap& out, const tma::TensorMap& phi,
-                            const PipeZArgs& a, cudaStream_t st) {
-  const size_t stage = (size_t)N * PipeCfg<N>::PZ * (SC ? 4 : 3);
-  const size_t sm = sizeof(float2) * (2 * N + 2 * stage);
-  cudaError_t e = set_smem(k_zpass_pipe<N, MODE, SC>, sm);
-  if (e != cudaSuccess) return e;
-  static int grid = 0;
-  constexpr int nt = zthreads<N, MODE>();
-  if (!grid) grid = pipe_grid(k_zpass_pipe<N, MODE, SC>, sm, nt);
-  const int ntiles = a.nyq_only ? PipeCfg<N>::NBLKZ + N - 1 : PipeCfg<N>::NBLKZ * N;
-  k_zpass_pipe<N, MODE, SC><<<capped(grid, ntiles, a.max_ctas), nt, sm, st>>>(in, out, phi, a);
-  return cudaGetLastError();
-}
-
-template <int MODE>
-cudaError_t launch_zpipe(const tma::TensorMap& in, const tma::TensorMap& out, const tma::TensorMap& phi,
-                         const PipeZArgs& a, cudaStream_t st) {
-  // a separate scalar region only when the potential is stored, or kept for
-  // the mean of the last two iterations
-  if constexpr (MODE == Z_NEWTON || MODE == Z_FINAL || MODE == Z_CURL) {
-    if (((MODE != Z_CURL) && a.nout > 3) || a.mean) return launch_zpipe_sc<MODE, true>(in, out, phi, a, st);
-  }
-  return launch_zpipe_sc<MODE, false>(in, out, phi, a, st);
-}
 }  // namespace
 
 cudaError_t CAT(mond_ypass_pipe_, MOND_N)(int dir, const tma::TensorMap& map, const passes::PipeYArgs& a,
@@ -137,85 +112,55 @@ cudaError_t CAT(mond_ypass_pipe_, MOND_N)(int dir, const tma::TensorMap& map, co
   return dir < 0 ? launch_ypipe<-1>(map, a, st) : launch_ypipe<+1>(map, a, st);
 }
 
-cudaError_t CAT(mond_zpass_pipe_, MOND_N)(int mode, const tma::TensorMap& in, const tma::TensorMap& out,
-                                          const tma::TensorMap& phi, const passes::PipeZArgs& a, cudaStream_t st) {
-  switch (mode) {
-    case Z_NEWTON: return launch_zpipe<Z_NEWTON>(in, out, phi, a, st);
-    case Z_CURL: return launch_zpipe<Z_CURL>(in, out, phi, a, st);
-    case Z_DIV: return launch_zpipe<Z_DIV>(in, out, phi, a, st);
-    case Z_FINAL: return launch_zpipe<Z_FINAL>(in, out, phi, a, st);
-    case Z_SMOOTH: return launch_zpipe<Z_SMOOTH>(in, out, phi, a, st);
-  }
-  return cudaErrorInvalidValue;
-}
-
 namespace {
 template <int KIND>
-cudaError_t launch_yfold(const tma::TensorMap& map4, const tma::TensorMap& mapc, const tma::TensorMap& mapp,
-                         const PipeYFArgs& a, cudaStream_t st) {
-  if constexpr (!fold_ok(N)) {
-    return cudaErrorInvalidValue;
-  } else {
-    const size_t sm = sizeof(float2) * (2 * N + 2 * (size_t)N * pipe_py(N));
-    cudaError_t e = set_smem(k_ypass_fold<N, KIND>, sm);
-    if (e != cudaSuccess) return e;
-    static int grid = 0;
-    if (!grid) grid = pipe_grid(k_ypass_fold<N, KIND>, sm, yf_threads(N));
-    const int nbf = (N / 2 + pipe_pyf(N)) / pipe_pyf(N), nbp = (N / 2 + pipe_py(N)) / pipe_py(N);
-    const int ntiles = nbf * N + nbp * N * a.nplain;
-    k_ypass_fold<N, KIND><<<capped(grid, ntiles, a.max_ctas), yf_threads(N), sm, st>>>(map4, mapc, mapp, a);
-    return cudaGetLastError();
-  }
+cudaError_t launch_yreg(const regpass::YRegArgs& a, int cap, cudaStream_t st) {
+  using G = regpass::YGeo<N, KIND>;
+  constexpr bool PAIR = KIND >= regpass::Y_FOLD;
+  const size_t sm = sizeof(float2) * (N + (PAIR ? N / 2 + 2 * G::SLOTS : G::SLOTS));
+  cudaError_t e = sm > 48 * 1024 ? set_smem(regpass::k_yreg<N, KIND>, sm) : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  const int ntiles = G::TILES * (a.nplain + (PAIR ? 1 : 0));
+  regpass::k_yreg<N, KIND><<<capped(ntiles, ntiles, cap), G::T, sm, st>>>(a, ntiles);
+  return cudaGetLastError();
 }
 
-template <int MODE, int SCK>
-cudaError_t launch_zfold_sc(const tma::TensorMap& in2, const tma::TensorMap& out2, const tma::TensorMap& phi,
-                            const PipeZArgs& a, cudaStream_t st) {
-  if constexpr (!fold_ok(N)) {
-    return cudaErrorInvalidValue;
-  } else {
-    const size_t R = (size_t)N * PipeCfg<N>::PZ;
-    const size_t stage = 2 * R + (SCK ? R : 0);
-    const size_t sm = sizeof(float2) * (2 * N + 2 * stage);
-    cudaError_t e = set_smem(k_zpass_fold<N, MODE, SCK>, sm);
-    if (e != cudaSuccess) return e;
-    static int grid = 0;
-    if (!grid) grid = pipe_grid(k_zpass_fold<N, MODE, SCK>, sm, 128);
-    const int nbr = MODE == Z_NEWTON ? PipeCfg<N>::NBLKZ : PipeCfg<N>::NBLKZ - 1;
-    const int ntiles = MODE == Z_NEWTON ? nbr * N : nbr * (N - 1);
-    k_zpass_fold<N, MODE, SCK><<<capped(grid, ntiles, a.max_ctas), 128, sm, st>>>(in2, out2, phi, a);
-    return cudaGetLastError();
-  }
-}
-
-template <int MODE>
-cudaError_t launch_zfold(const tma::TensorMap& in2, const tma::TensorMap& out2, const tma::TensorMap& phi,
-                         const PipeZArgs& a, cudaStream_t st) {
-  // a scalar region for the mean of the last two iterations; its inverse z
-  // transform too when the potential is stored
-  if (MODE != Z_CURL && a.nout > 3) return launch_zfold_sc<MODE, 2>(in2, out2, phi, a, st);
-  if (a.mean) return launch_zfold_sc<MODE, 1>(in2, out2, phi, a, st);
-  return launch_zfold_sc<MODE, 0>(in2, out2, phi, a, st);
+template <int MODE, bool FOLD, bool PHI>
+cudaError_t launch_zreg(const regpass::ZRegArgs& a, int cap, cudaStream_t st) {
+  using G = regpass::Geo<N>;
+  const size_t sm = regpass::ZCfg<N, MODE, FOLD, PHI>::smem();
+  cudaError_t e = sm > 48 * 1024 ? set_smem(regpass::k_zreg<N, MODE, FOLD, PHI>, sm) : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  regpass::k_zreg<N, MODE, FOLD, PHI><<<capped(G::TILES, G::TILES, cap), G::T, sm, st>>>(a, G::TILES);
+  return cudaGetLastError();
 }
 }  // namespace
 
-cudaError_t CAT(mond_ypass_fold_, MOND_N)(int kind, const tma::TensorMap& map4, const tma::TensorMap& mapc,
-                                          const tma::TensorMap& mapp, const passes::PipeYFArgs& a, cudaStream_t st) {
+cudaError_t CAT(mond_yreg_, MOND_N)(int kind, const regpass::YRegArgs& a, int cap, cudaStream_t st) {
   switch (kind) {
-    case YF_FOLD: return launch_yfold<YF_FOLD>(map4, mapc, mapp, a, st);
-    case YF_CURL: return launch_yfold<YF_CURL>(map4, mapc, mapp, a, st);
-    case YF_GRADN: return launch_yfold<YF_GRADN>(map4, mapc, mapp, a, st);
-    case YF_GRAD: return launch_yfold<YF_GRAD>(map4, mapc, mapp, a, st);
+    case regpass::Y_FWD: return launch_yreg<regpass::Y_FWD>(a, cap, st);
+    case regpass::Y_INV: return launch_yreg<regpass::Y_INV>(a, cap, st);
+    case regpass::Y_FOLD: return launch_yreg<regpass::Y_FOLD>(a, cap, st);
+    case regpass::Y_CURL: return launch_yreg<regpass::Y_CURL>(a, cap, st);
+    case regpass::Y_GRADN: return launch_yreg<regpass::Y_GRADN>(a, cap, st);
+    case regpass::Y_GRAD: return launch_yreg<regpass::Y_GRAD>(a, cap, st);
   }
   return cudaErrorInvalidValue;
 }
 
-cudaError_t CAT(mond_zpass_fold_, MOND_N)(int mode, const tma::TensorMap& in2, const tma::TensorMap& out2,
-                                          const tma::TensorMap& phi, const passes::PipeZArgs& a, cudaStream_t st) {
+cudaError_t CAT(mond_zreg_, MOND_N)(int mode, bool fold, bool phi, const regpass::ZRegArgs& a, int cap,
+                                    cudaStream_t st) {
   switch (mode) {
-    case Z_NEWTON: return launch_zfold<Z_NEWTON>(in2, out2, phi, a, st);
-    case Z_CURL: return launch_zfold<Z_CURL>(in2, out2, phi, a, st);
-    case Z_FINAL: return launch_zfold<Z_FINAL>(in2, out2, phi, a, st);
+    case Z_NEWTON:
+      if (fold) return phi ? launch_zreg<Z_NEWTON, true, true>(a, cap, st) : launch_zreg<Z_NEWTON, true, false>(a, cap, st);
+      return phi ? launch_zreg<Z_NEWTON, false, true>(a, cap, st) : launch_zreg<Z_NEWTON, false, false>(a, cap, st);
+    case Z_CURL:
+      return fold ? launch_zreg<Z_CURL, true, false>(a, cap, st) : launch_zreg<Z_CURL, false, false>(a, cap, st);
+    case Z_FINAL:
+      if (fold) return phi ? launch_zreg<Z_FINAL, true, true>(a, cap, st) : launch_zreg<Z_FINAL, true, false>(a, cap, st);
+      return phi ? launch_zreg<Z_FINAL, false, true>(a, cap, st) : launch_zreg<Z_FINAL, false, false>(a, cap, st);
+    case Z_DIV: return launch_zreg<Z_DIV, false, false>(a, cap, st);
+    case Z_SMOOTH: return launch_zreg<Z_SMOOTH, false, false>(a, cap, st);
   }
   return cudaErrorInvalidValue;
 }
