@@ -374,6 +374,9 @@ __device__ __forceinline__ void xfft(float2* buf, int nc, const float2* tw, int 
   if (c < nc) fftk::fft_c<C::H, DIR, C::L, 1, NTX>(buf + c * TILE, C::LP, 1, TILE, tw, 2, tid);
 }
 
+// The density pass and the passes of the incremental solve (the others are
+// those of xreg.cuh; the density pass in registers was slower, 0.105 against
+// 0.089 ms at 256: its int64 loads want more threads).
 template <int N, int MODE>
 __global__ void __launch_bounds__(NTX) k_xpass(XArgs a, int64_t nlines) {
   using C = XCfg<N>;
@@ -384,25 +387,17 @@ __global__ void __launch_bounds__(NTX) k_xpass(XArgs a, int64_t nlines) {
   const int tid = threadIdx.x;
   const int64_t line0 = (int64_t)blockIdx.x * C::L;
   for (int i = tid; i < N; i += NTX) tw[i] = a.tw[i];
-  const int nc = (MODE == X_RHO || MODE == X_DRHO) ? 1 : a.ncomp;
+  constexpr bool INC = MODE == X_DNU_FIRST || MODE == X_DNU || MODE == X_DMU;  // three components, C2R first
+  static_assert(INC || MODE == X_RHO || MODE == X_DRHO, "modes of k_xpass");
+  constexpr int nc = INC ? 3 : 1;
 
-  constexpr bool INC = (MODE == X_DNU_FIRST || MODE == X_DNU || MODE == X_DMU);  // incremental, 3 components
-  constexpr bool INV = (MODE == X_NU_FIRST || MODE == X_NU || MODE == X_MU || MODE == X_INV || INC);
-  constexpr bool FWD = (MODE == X_RHO || MODE == X_NU_FIRST || MODE == X_NU || MODE == X_MU || MODE == X_FWD ||
-                        MODE == X_NU_REAL || MODE == X_DRHO || INC);
-
-  if (tid == 0) {
+  if (tid == 0 && INC) {
     // the real-space planes the pointwise stage reads, brought into L2 while
     // the spectral tile is loaded and transformed (L lines: contiguous)
     const uint32_t rb = (uint32_t)(C::L * N * sizeof(float));
     const int64_t r0 = line0 * N;
     for (int c = 0; c < 3; c++) {
       const int64_t o = (int64_t)c * N * N * N + r0;
-      if constexpr (MODE == X_NU || MODE == X_MU || MODE == X_NU_REAL) tma::prefetch_l2(a.gN + o, rb);
-      if constexpr (MODE == X_NU_FIRST || MODE == X_NU_REAL)
-        if (a.H0) tma::prefetch_l2(a.H0 + o, rb);
-      if constexpr (MODE == X_NU)
-        if (a.Hs_out && a.red) tma::prefetch_l2(a.Hs_out + o, rb);
       if constexpr (MODE == X_DNU_FIRST || MODE == X_DNU) {
         tma::prefetch_l2(a.gN + o, rb);
         tma::prefetch_l2(a.H0 + o, rb);
@@ -411,7 +406,7 @@ __global__ void __launch_bounds__(NTX) k_xpass(XArgs a, int64_t nlines) {
       if constexpr (MODE == X_DMU) tma::prefetch_l2(a.gM0 + o, rb);
     }
   }
-  if constexpr (INV) {
+  if constexpr (INC) {
     for (int c = 0; c < nc; c++) x_load_spec<N>(buf + c * TILE, a.spec + c * a.pstride, line0, tid);
     tma::async_wait_all();
     __syncthreads();
@@ -421,7 +416,6 @@ __global__ void __launch_bounds__(NTX) k_xpass(XArgs a, int64_t nlines) {
 
   // Pointwise stage on real samples: point (j, l) holds x[2j], x[2j+1] of line l.
   const int64_t rbase = line0 * N;  // real index of the first sample of the tile
-  float sq_dh = 0.f, sq_gn = 0.f;
   bool bad = false;
   if constexpr (MODE == X_RHO) {
     // the density: all of a thread's accumulator loads in flight at once, then the rule
@@ -524,133 +518,14 @@ __global__ void __launch_bounds__(NTX) k_xpass(XArgs a, int64_t nlines) {
         }
       }
       for (int c = 0; c < 3; c++) p0[c * TILE] = make_float2(v[c][0], v[c][1]);
-    } else if constexpr (MODE == X_FWD) {
-      for (int c = 0; c < nc; c++) p0[c * TILE] = *reinterpret_cast<const float2*>(a.real_in + (int64_t)c * N * N * N + ri);
-      if (a.ext_axis1) {
-        const float2 e = dipole2<N>(a, line0 + l, 2 * j);
-        p0[0].x += e.x;
-        p0[0].y += e.y;
-      }
-    } else if constexpr (MODE == X_INV) {
-      for (int c = 0; c < nc; c++) {
-        float2 v = p0[c * TILE];
-        bad |= !(isfinite(v.x) && isfinite(v.y));
-        float2* dst = reinterpret_cast<float2*>(a.real_out + (int64_t)c * N * N * N + ri);
-        if (a.accumulate) {
-          const float2 o = *dst;
-          v.x += o.x;
-          v.y += o.y;
-        }
-        *dst = v;
-        if (a.real_out2) *reinterpret_cast<float2*>(a.real_out2 + (int64_t)c * N * N * N + ri) = v;
-      }
-    } else {
-      // three components, two samples each
-      float v[3][2], gn[3][2];
-      if constexpr (MODE != X_NU_REAL) {
-        for (int c = 0; c < 3; c++) {
-          float2 t = p0[c * TILE];
-          v[c][0] = t.x;
-          v[c][1] = t.y;
-        }
-      }
-      if constexpr (MODE == X_NU_REAL) {
-        // F = g_N + H0 from the stored Newton field
-        for (int c = 0; c < 3; c++) {
-          float2 t = *reinterpret_cast<const float2*>(a.gN + (int64_t)c * N * N * N + ri);
-          float2 h0 = a.H0 ? *reinterpret_cast<const float2*>(a.H0 + (int64_t)c * N * N * N + ri)
-                           : make_float2(0.f, 0.f);
-          gn[c][0] = t.x;
-          gn[c][1] = t.y;
-          v[c][0] = t.x + h0.x;
-          v[c][1] = t.y + h0.y;
-        }
-      } else if constexpr (MODE == X_NU_FIRST) {
-        // input is g_N; store it; F = g_N + H0
-        for (int c = 0; c < 3; c++) {
-          *reinterpret_cast<float2*>(a.gN_out + (int64_t)c * N * N * N + ri) = make_float2(v[c][0], v[c][1]);
-          gn[c][0] = v[c][0];
-          gn[c][1] = v[c][1];
-          float2 h0 = a.H0 ? *reinterpret_cast<const float2*>(a.H0 + (int64_t)c * N * N * N + ri)
-                           : make_float2(0.f, 0.f);
-          v[c][0] += h0.x;
-          v[c][1] += h0.y;
-        }
-      } else {
-        for (int c = 0; c < 3; c++) {
-          float2 t = *reinterpret_cast<const float2*>(a.gN + (int64_t)c * N * N * N + ri);
-          gn[c][0] = t.x;
-          gn[c][1] = t.y;
-        }
-      }
-      if constexpr (MODE == X_MU) {
-        if (a.gM_out)
-          for (int c = 0; c < 3; c++)
-            *reinterpret_cast<float2*>(a.gM_out + (int64_t)c * N * N * N + ri) = make_float2(v[c][0], v[c][1]);
-      }
-      if constexpr (MODE == X_NU) {
-        // input is H after the divergence-free projection
-        if (a.Hs_out) {
-          for (int c = 0; c < 3; c++) {
-            float* hp = a.Hs_out + (int64_t)c * N * N * N + ri;
-            if (a.red) {
-              float2 old = *reinterpret_cast<const float2*>(hp);
-              float d0 = v[c][0] - old.x, d1 = v[c][1] - old.y;
-              sq_dh += d0 * d0 + d1 * d1;
-              sq_gn += gn[c][0] * gn[c][0] + gn[c][1] * gn[c][1];
-            }
-            *reinterpret_cast<float2*>(hp) = make_float2(v[c][0], v[c][1]);
-          }
-        }
-        for (int c = 0; c < 3; c++) {
-          v[c][0] += gn[c][0];
-          v[c][1] += gn[c][1];
-        }
-      }
-      for (int e = 0; e < 2; e++) {
-        float m2 = v[0][e] * v[0][e] + v[1][e] * v[1][e] + v[2][e] * v[2][e];
-        float f;
-        if (a.mu_kind == 0) {
-          // deep MOND, from the hardware reciprocal square root (a few ulp, no
-          // IEEE divide or square root): nu = sqrt(a0 / |F|) = sqrt(a0) (m2)^-1/4,
-          // mu |g| / a0 with |g| = m2 / sqrt(m2); 0 at zero field
-          const float r = m2 > 0.f ? rsqrtf(m2) : 0.f;  // 1 / |v|
-          if constexpr (MODE == X_MU) f = m2 * r * a.inv_a0;
-          else f = a.sqrt_a0 * (r * rsqrtf(r > 0.f ? r : 1.f)) * (r > 0.f ? 1.f : 0.f);
-        } else {
-          const float mag = sqrtf(m2);
-          if constexpr (MODE == X_MU) f = mu_factor(a.mu_kind, mag, a.a0);
-          else f = nu_factor(a.mu_kind, mag, a.a0);
-        }
-        for (int c = 0; c < 3; c++) {
-          float o = f * v[c][e];
-          if constexpr (MODE == X_MU) o -= gn[c][e];  // H = F - g_N
-          v[c][e] = o;
-        }
-        bad |= !isfinite(m2);
-      }
-      for (int c = 0; c < 3; c++) p0[c * TILE] = make_float2(v[c][0], v[c][1]);
     }
   }
   if (bad) set_status(a.status, ST_NAN);
-  if (MODE == X_NU && a.red && a.Hs_out) {
-    // per-CTA partial sums of |dH|^2 and |g_N|^2
-    for (int o = 16; o > 0; o >>= 1) {
-      sq_dh += __shfl_xor_sync(0xffffffffu, sq_dh, o);
-      sq_gn += __shfl_xor_sync(0xffffffffu, sq_gn, o);
-    }
-    if ((tid & 31) == 0) {
-      atomicAdd(a.red, (double)sq_dh);
-      atomicAdd(a.red + 1, (double)sq_gn);
-    }
-  }
 
-  if constexpr (FWD) {
-    __syncthreads();
-    xfft<N, -1>(buf, nc, tw, tid);
-    x_post_r2c<N>(buf, nc, tw, tid);
-    for (int c = 0; c < nc; c++) x_store_spec<N>(buf + c * TILE, a.spec + c * a.pstride, line0, tid);
-  }
+  __syncthreads();
+  xfft<N, -1>(buf, nc, tw, tid);
+  x_post_r2c<N>(buf, nc, tw, tid);
+  for (int c = 0; c < nc; c++) x_store_spec<N>(buf + c * TILE, a.spec + c * a.pstride, line0, tid);
 }
 
 // ---------------------------------------------------------------------------

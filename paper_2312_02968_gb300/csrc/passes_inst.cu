@@ -2,6 +2,7 @@
 // N = MOND_N (this file is compiled once per supported size, in parallel).
 #include "launch.h"
 #include "regpass.cuh"
+#include "xreg.cuh"
 
 #ifndef MOND_N
 #error "compile with -DMOND_N=<size>"
@@ -22,12 +23,22 @@ size_t z_smem(int ntiles) { return sizeof(float2) * (2 * N + (size_t)ntiles * N 
 
 template <int MODE>
 cudaError_t launch_x(const XArgs& a, cudaStream_t st) {
-  int nc = (MODE == X_RHO || MODE == X_DRHO) ? 1 : a.ncomp;
-  size_t sm = x_smem(nc);
-  cudaError_t e = set_smem(k_xpass<N, MODE>, x_smem(4));
+  const size_t sm = x_smem((MODE == X_RHO || MODE == X_DRHO) ? 1 : 3);
+  cudaError_t e = set_smem(k_xpass<N, MODE>, sm);
   if (e != cudaSuccess) return e;
   int64_t nlines = (int64_t)N * N;
   k_xpass<N, MODE><<<(unsigned)(nlines / XCfg<N>::L), NTX, sm, st>>>(a, nlines);
+  return cudaGetLastError();
+}
+
+template <int MODE>
+cudaError_t launch_xreg(const XArgs& a, cudaStream_t st) {
+  using X = xreg::Geo<N>;
+  constexpr size_t sm = xreg::smem_bytes<N, MODE>();
+  cudaError_t e = sm > 48 * 1024 ? set_smem(xreg::k_xreg<N, MODE>, sm) : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  const dim3 grid(N * N / X::LINES, xreg::ncomp_of(MODE) == 3 ? 1 : a.ncomp);
+  xreg::k_xreg<N, MODE><<<grid, 32 * xreg::WARPS, sm, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -48,12 +59,12 @@ cudaError_t launch_z(const ZArgs& a, cudaStream_t st) {
 cudaError_t CAT(mond_xpass_, MOND_N)(int mode, const passes::XArgs& a, cudaStream_t st) {
   switch (mode) {
     case X_RHO: return launch_x<X_RHO>(a, st);
-    case X_NU_FIRST: return launch_x<X_NU_FIRST>(a, st);
-    case X_NU: return launch_x<X_NU>(a, st);
-    case X_MU: return launch_x<X_MU>(a, st);
-    case X_INV: return launch_x<X_INV>(a, st);
-    case X_FWD: return launch_x<X_FWD>(a, st);
-    case X_NU_REAL: return launch_x<X_NU_REAL>(a, st);
+    case X_NU_FIRST: return launch_xreg<X_NU_FIRST>(a, st);
+    case X_NU: return launch_xreg<X_NU>(a, st);
+    case X_MU: return launch_xreg<X_MU>(a, st);
+    case X_INV: return launch_xreg<X_INV>(a, st);
+    case X_FWD: return launch_xreg<X_FWD>(a, st);
+    case X_NU_REAL: return launch_xreg<X_NU_REAL>(a, st);
     case X_DRHO: return launch_x<X_DRHO>(a, st);
     case X_DNU_FIRST: return launch_x<X_DNU_FIRST>(a, st);
     case X_DNU: return launch_x<X_DNU>(a, st);
