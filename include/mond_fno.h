@@ -76,6 +76,13 @@ int mond_fno_loss(int64_t count, const float* y, const float* t, float* dy, floa
 int mond_fno_adam(int64_t count, float* params, float* grad, float* m, float* v, float lr, float beta1, float beta2,
                   float eps, int step, float clip_norm, double* scratch, void* stream);
 
+/* mond_fno_adam that also leaves the bfloat16 copy of the new parameters
+ * (mond_fno_cast of them) in params_bf16 (count values; NULL: no copy), in the
+ * same pass over memory. */
+int mond_fno_adam_cast(int64_t count, float* params, float* grad, float* m, float* v, float lr, float beta1,
+                       float beta2, float eps, int step, float clip_norm, double* scratch, uint16_t* params_bf16,
+                       void* stream);
+
 /* Network input from a fine Newtonian field: g_N [3][N^3] (N = f n) is
  * averaged over f^3 blocks to the coarse grid and normalised: x [4][n^3].
  * scale_out points to 4 device floats, 8-byte aligned: scale_out[0] = s (the

@@ -95,12 +95,11 @@ class FNO:
 
     def adam(self, lr, b1=0.9, b2=0.999, eps=1e-8, clip=0.0):
         """One Adam step; clip > 0 caps the gradient norm; a non-finite
-        gradient is dropped."""
+        gradient is dropped. The bfloat16 copy follows in the same pass."""
         self.steps += 1
-        _check(lib().mond_fno_adam(self.count, _p(self.params), _p(self.grad), _p(self.m), _p(self.v), float(lr),
-                                   float(b1), float(b2), float(eps), self.steps, float(clip), _p(self.adam_scratch),
-                                   self._st), "adam")
-        self.cast()
+        _check(lib().mond_fno_adam_cast(self.count, _p(self.params), _p(self.grad), _p(self.m), _p(self.v), float(lr),
+                                        float(b1), float(b2), float(eps), self.steps, float(clip),
+                                        _p(self.adam_scratch), _p(self.params_bf16), self._st), "adam")
 
     # ----------------------------------------------------------- training
     def train(self, xs, ts, epochs: int, batch: int, lr: float, seed: int = 0, lr_final: float | None = None,
