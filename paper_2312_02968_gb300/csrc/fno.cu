@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "../../include/mond_fno.h"
 #include "internal.h"
@@ -50,23 +51,6 @@ bool make_shape(const mond_fno_shape& s, Shape* o) {
   return true;
 }
 
-// Tables of the truncated transforms, rebuilt by every forward/backward call:
-//   fx  [n][SXF]   x-forward: (cos, -sin)(2 pi kx x/n) for kx < M, zero padded
-//   ix  [2M][SXI]  x-inverse, weight a(kx)/V: rows (cos, -sin)(2 pi kx x/n)
-//   ixa [2M][SXI]  the same with weight 1 (adjoint of the x-forward)
-//   tf  [2M][n]    forward along y or z: e^{-2 pi i f(p) q / n}
-//   ti  [n][2M]    inverse along y or z: e^{+2 pi i f(q) p / n}
-// SXF = 16 ceil(M/8) and SXI = 16 ceil(n/16) floats (zero beyond the data).
-struct Tabs {
-  float* fx;
-  float* ix;
-  float* ixa;
-  float2* tf;
-  float2* ti;
-};
-__host__ __device__ inline int sxf(int M) { return 16 * ((M + 7) / 8); }
-__host__ __device__ inline int sxi(int n) { return 16 * ((n + 15) / 16); }
-
 // Workspace layout for one sample.
 struct Work {
   float* v;      // (L+1) x C x V activations (v_0 .. v_L)
@@ -78,7 +62,6 @@ struct Work {
   float* dv;     // C x V
   float* dv2;    // C x V
   float* dz;     // C x V
-  Tabs tab;      // transform tables
 };
 
 size_t carve(const Shape& s, char* base, Work* w) {
@@ -99,11 +82,6 @@ size_t carve(const Shape& s, char* base, Work* w) {
   t.dv = (float*)take(sizeof(float) * CV);
   t.dv2 = (float*)take(sizeof(float) * CV);
   t.dz = (float*)take(sizeof(float) * CV);
-  t.tab.fx = (float*)take(sizeof(float) * s.n * 64);
-  t.tab.ix = (float*)take(sizeof(float) * 2 * s.M * 64);
-  t.tab.ixa = (float*)take(sizeof(float) * 2 * s.M * 64);
-  t.tab.tf = (float2*)take(sizeof(float2) * 2 * s.M * s.n);
-  t.tab.ti = (float2*)take(sizeof(float2) * 2 * s.M * s.n);
   if (w) *w = t;
   return off;
 }
@@ -111,24 +89,6 @@ size_t carve(const Shape& s, char* base, Work* w) {
 __device__ __forceinline__ float bf(const uint16_t* p, int64_t i) {
   return __bfloat162float(__ushort_as_bfloat16(p[i]));
 }
-
-// 16-byte asynchronous copy global -> shared; groups complete in order.
-__device__ __forceinline__ void cp16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int PENDING>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
-
-// e^{sign 2 pi i m / n} with exact argument reduction of m modulo n.
-__device__ __forceinline__ float2 cis(int64_t m, int n, float sign) {
-  int r = (int)(((m % n) + n) % n);
-  float sn, cs;
-  sincospif(2.0f * (float)r / (float)n, &sn, &cs);
-  return make_float2(cs, sign * sn);
-}
-__device__ __forceinline__ int sfreq(int i, int M) { return i < M ? i : i - 2 * M; }
 
 // out[o][v] = sum_i W[o][i] in[i][v] (+ b[o]); transpose uses W[i][o].
 // CMAX >= Cin: the input channels sit in registers, the weights in shared
@@ -309,311 +269,18 @@ __global__ void k_wgrad(const float* dout, int Cout, const float* in, int Cin, i
   }
 }
 
+// gelu in the tanh form, (1 + tanh u)/2 as the logistic function of 2u: no
+// cancellation at negative u, and one exponential and one division instead
+// of tanhf's two branches (it was a third of the inverse transform's time).
 __device__ __forceinline__ float gelu_t(float z, float* dgdz) {
   const float k0 = 0.7978845608028654f, k1 = 0.044715f;
   const float u = k0 * (z + k1 * z * z * z);
-  const float th = tanhf(u);
-  if (dgdz) *dgdz = 0.5f * (1.f + th) + 0.5f * z * (1.f - th * th) * k0 * (1.f + 3.f * k1 * z * z);
-  return 0.5f * z * (1.f + th);
+  const float t = expf(fminf(-2.f * u, 80.f)), s = 1.f / (1.f + t);
+  if (dgdz) *dgdz = s + z * (t * s * s) * (2.f * k0) * (1.f + 3.f * k1 * z * z);
+  return z * s;
 }
 
-__global__ void k_tables(int n, int M, float invV, Tabs t) {
-  const int SXF = sxf(M), SXI = sxi(n);
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * SXF; e += gridDim.x * blockDim.x) {
-    const int x = e / SXF, j = e % SXF, kx = j / 2;
-    float v = 0.f;
-    if (kx < M) {
-      const float2 w = cis((int64_t)kx * x, n, -1.f);
-      v = (j & 1) ? w.y : w.x;
-    }
-    t.fx[e] = v;
-  }
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 2 * M * SXI; e += gridDim.x * blockDim.x) {
-    const int j = e / SXI, x = e % SXI, kx = j / 2;
-    float v = 0.f;
-    if (x < n) {
-      const float2 w = cis((int64_t)kx * x, n, -1.f);
-      v = (j & 1) ? w.y : w.x;
-    }
-    t.ixa[e] = v;
-    t.ix[e] = v * (kx == 0 ? 1.f : 2.f) * invV;
-  }
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 2 * M * n; e += gridDim.x * blockDim.x) {
-    const int p = e / n, q = e % n;
-    t.tf[e] = cis((int64_t)sfreq(p, M) * q, n, -1.f);
-    const int pp = e / (2 * M), qq = e % (2 * M);
-    t.ti[e] = cis((int64_t)sfreq(qq, M) * pp, n, 1.f);
-  }
-}
-
-// Forward transform of (c, z) planes along x and y, fused, n <= 64, M <= 32:
-// the n x n real plane is staged in shared memory and transformed along x to
-// n x M complex, X[y][kx] = sum_x v[y][x] e^{-2 pi i kx x/n}, then along y,
-// out[p][kx] = sum_y e^{-2 pi i f(p) y/n} X[y][kx], p < 2M.
-// x: lane j owns output float j of a row (re/im of kx = j/2) and keeps its
-// table column in registers; the plane row is read as float4 broadcasts.
-// y: lane p owns an output row; X is read as broadcasts. Persistent CTAs
-// loop over planes, so the tables are read once per CTA.
-__host__ __device__ inline int round4(int x) { return (x + 3) & ~3; }
-size_t smem_xy_fwd(int n, int M) {
-  return sizeof(float) * ((size_t)2 * n * n + (size_t)n * round4(2 * M) + (size_t)2 * M * M * 2) +
-         sizeof(float2) * (size_t)2 * M * (n + 1);
-}
-template <int NX>  // n <= NX
-__global__ void __launch_bounds__(256, 2) k_xy_fwd(const float* __restrict__ v, float2* __restrict__ out,
-                                                const float* __restrict__ fx, const float2* __restrict__ tf, int n,
-                                                int M, int64_t nplanes) {
-  extern __shared__ __align__(16) float smf[];
-  const int M2 = 2 * M, XS = round4(M2), SXF = sxf(M);
-  float* sP = smf;                                          // 2 * n * n: the plane, double buffered
-  float* sX = sP + 2 * n * n;                               // n * XS
-  float2* sO = reinterpret_cast<float2*>(sX + n * XS);      // M2 * M
-  float2* sY = sO + M2 * M;                                 // M2 * (n + 1)
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float tx[NX];
-#pragma unroll
-  for (int x = 0; x < NX; x++) tx[x] = (x < n && lane < M2) ? fx[x * SXF + lane] : 0.f;
-  for (int e = tid; e < M2 * n; e += blockDim.x) sY[(e / n) * (n + 1) + e % n] = tf[e];
-  const int KPG = (M + 7) / 8;  // kx per warp in the y stage
-  // the next plane is copied in while this one is transformed
-  auto fetch = [&](int64_t plane, float* dst) {
-    const float* src = v + plane * n * n;
-    for (int e = tid; e < n * n / 4; e += blockDim.x) cp16(dst + 4 * e, src + 4 * e);
-  };
-  if ((int64_t)blockIdx.x < nplanes) fetch(blockIdx.x, sP);
-  cp_commit();
-  int it = 0;
-  for (int64_t plane = blockIdx.x; plane < nplanes; plane += gridDim.x, it++) {
-    const int64_t nxt = plane + gridDim.x;
-    if (nxt < nplanes) fetch(nxt, sP + ((it + 1) & 1) * n * n);
-    cp_commit();
-    cp_wait<1>();  // this plane's group is complete
-    __syncthreads();
-    const float4* sP4 = reinterpret_cast<const float4*>(sP + (it & 1) * n * n);
-    for (int r = warp; r < n; r += 16) {
-      const int r2 = r + 8;
-      const float4* a0 = sP4 + r * (n / 4);
-      const float4* a1 = sP4 + (r2 < n ? r2 : r) * (n / 4);
-      float acc0 = 0.f, acc1 = 0.f;
-#pragma unroll
-      for (int q = 0; q < NX / 4; q++) {
-        if (4 * q < n) {
-          const float4 u = a0[q], w = a1[q];
-          acc0 = fmaf(u.x, tx[4 * q], fmaf(u.y, tx[4 * q + 1], fmaf(u.z, tx[4 * q + 2], fmaf(u.w, tx[4 * q + 3], acc0))));
-          acc1 = fmaf(w.x, tx[4 * q], fmaf(w.y, tx[4 * q + 1], fmaf(w.z, tx[4 * q + 2], fmaf(w.w, tx[4 * q + 3], acc1))));
-        }
-      }
-      if (lane < M2) {
-        sX[r * XS + lane] = acc0;
-        if (r2 < n) sX[r2 * XS + lane] = acc1;
-      }
-    }
-    __syncthreads();
-    if (lane < M2) {
-      const float2* t = sY + lane * (n + 1);
-      float2 acc[4];
-#pragma unroll
-      for (int k = 0; k < 4; k++) acc[k] = make_float2(0.f, 0.f);
-      for (int y = 0; y < n; y++) {
-        const float2 w = t[y];
-        const float* xr = sX + y * XS;
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-          const int kx = warp * KPG + k;
-          if (k < KPG && kx < M) {
-            const float a = xr[2 * kx], b = xr[2 * kx + 1];
-            acc[k].x = fmaf(w.x, a, fmaf(-w.y, b, acc[k].x));
-            acc[k].y = fmaf(w.x, b, fmaf(w.y, a, acc[k].y));
-          }
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const int kx = warp * KPG + k;
-        if (k < KPG && kx < M) sO[lane * M + kx] = acc[k];
-      }
-    }
-    __syncthreads();
-    float2* o = out + plane * M2 * M;
-    for (int e = tid; e < M2 * M; e += blockDim.x) o[e] = sO[e];
-  }
-}
-
-// Inverse of k_xy_fwd for planes, fused: in [2M][M] complex -> along y,
-// X[y][kx] = sum_p e^{+2 pi i f(p) y/n} in[p][kx], then along x to real,
-// z[y][x] += sum_j X_j[y] tab[j][x] over the 2M real parts (the table carries
-// a(kx)/V or 1), then v = gelu(z) (act 1), v = z (act 2) or nothing.
-// y: lane = y; x: thread = x with its table column in registers.
-size_t smem_xy_inv(int n, int M) {
-  return sizeof(float) * ((size_t)n * (round4(2 * M) + 4)) +
-         sizeof(float2) * ((size_t)n * (2 * M + 1) + (size_t)2 * 2 * M * M);
-}
-template <int NX, int MX>  // n <= NX, 2M <= MX
-__global__ void __launch_bounds__(256, 2) k_xy_inv(const float2* __restrict__ in, float* __restrict__ z,
-                                                float* __restrict__ v, const float* __restrict__ tab,
-                                                const float2* __restrict__ ti, int n, int M, int act,
-                                                int64_t nplanes) {
-  extern __shared__ __align__(16) float smf[];
-  const int M2 = 2 * M, XS = round4(M2) + 4, SXI = sxi(n);  // XS: 4-way write conflicts at most
-  float* sX = smf;                                          // n * XS
-  float2* sTi = reinterpret_cast<float2*>(sX + n * XS);     // n * (M2 + 1)
-  float2* sI = sTi + n * (M2 + 1);                          // 2 * M2 * M: the input plane, double buffered
-  const int tid = threadIdx.x;
-  const int xl = tid & 63, grp = tid >> 6;  // x stage: column x, row group (4 groups)
-  float tt[MX];
-#pragma unroll
-  for (int j = 0; j < MX; j++) tt[j] = (j < M2 && xl < n) ? tab[j * SXI + xl] : 0.f;
-  for (int e = tid; e < n * M2; e += blockDim.x) sTi[(e / M2) * (M2 + 1) + e % M2] = ti[e];
-  for (int e = tid; e < n * XS; e += blockDim.x) sX[e] = 0.f;  // the row padding is read (times 0) below
-  const int KPG = (M + 3) / 4;  // kx per group in the y stage
-  // the next input plane is copied in while this one is transformed
-  auto fetch = [&](int64_t plane, float2* dst) {
-    const float2* src = in + plane * M2 * M;
-    for (int e = tid; e < M2 * M / 2; e += blockDim.x) cp16(dst + 2 * e, src + 2 * e);
-  };
-  if ((int64_t)blockIdx.x < nplanes) fetch(blockIdx.x, sI);
-  cp_commit();
-  int it = 0;
-  for (int64_t plane = blockIdx.x; plane < nplanes; plane += gridDim.x, it++) {
-    const int64_t nxt = plane + gridDim.x;
-    if (nxt < nplanes) fetch(nxt, sI + ((it + 1) & 1) * M2 * M);
-    cp_commit();
-    cp_wait<1>();
-    __syncthreads();
-    const float2* sIc = sI + (it & 1) * M2 * M;
-    if (xl < n) {
-      const float2* t = sTi + xl * (M2 + 1);  // row y = xl of the inverse table
-      float2 acc[8];
-#pragma unroll
-      for (int k = 0; k < 8; k++) acc[k] = make_float2(0.f, 0.f);
-      for (int p = 0; p < M2; p++) {
-        const float2 w = t[p];
-        const float2* ir = sIc + p * M;
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-          const int kx = grp * KPG + k;
-          if (k < KPG && kx < M) {
-            const float2 a = ir[kx];
-            acc[k].x = fmaf(w.x, a.x, fmaf(-w.y, a.y, acc[k].x));
-            acc[k].y = fmaf(w.x, a.y, fmaf(w.y, a.x, acc[k].y));
-          }
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 8; k++) {
-        const int kx = grp * KPG + k;
-        if (k < KPG && kx < M) {
-          sX[xl * XS + 2 * kx] = acc[k].x;
-          sX[xl * XS + 2 * kx + 1] = acc[k].y;
-        }
-      }
-    }
-    __syncthreads();
-    if (xl < n) {
-      float* zp = z + plane * n * n;
-      float* vp = v ? v + plane * n * n : nullptr;
-      // all of this thread's z values are requested before any is used
-      float zr[NX / 4];
-#pragma unroll
-      for (int k = 0; k < NX / 4; k++) {
-        const int y = grp + 4 * k;
-        zr[k] = y < n ? zp[(int64_t)y * n + xl] : 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < NX / 4; k++) {
-        const int y = grp + 4 * k;
-        if (y < n) {
-          const float4* xr = reinterpret_cast<const float4*>(sX + y * XS);
-          float acc = 0.f;
-#pragma unroll
-          for (int q = 0; q < MX / 4; q++) {
-            if (4 * q < M2) {
-              const float4 u = xr[q];
-              acc = fmaf(u.x, tt[4 * q],
-                         fmaf(u.y, tt[4 * q + 1], fmaf(u.z, tt[4 * q + 2], fmaf(u.w, tt[4 * q + 3], acc))));
-            }
-          }
-          const float zz = zr[k] + acc;
-          const int64_t i = (int64_t)y * n + xl;
-          zp[i] = zz;
-          if (act == 1) vp[i] = gelu_t(zz, nullptr);
-          else if (act == 2) vp[i] = zz;
-        }
-      }
-    }
-  }
-}
-
-// Complex contraction along a middle axis: out[b][p][i] = sum_q T[p][q] in[b][q][i]
-// (P, Q <= 64). Tiles of 16 columns i; a thread owns one column and the
-// rows p = p0, p0 + 16, ...; T stays in shared memory (row stride Q + 1).
-// Persistent CTAs: T is read once per CTA, and the next tile is copied in
-// (asynchronously, double buffered) while this one is contracted.
-constexpr int AXI = 16;
-__global__ void __launch_bounds__(256) k_axis(const float2* __restrict__ in, float2* __restrict__ out,
-                                              const float2* __restrict__ T, int64_t B, int P, int Q, int I) {
-  extern __shared__ __align__(16) float2 sma[];
-  const int QS = Q + 1;
-  float2* sT = sma;                                      // P * QS
-  float2* sIn = sma + ((P * QS + 1) & ~1);               // 2 * Q * AXI, 16-byte aligned
-  for (int e = threadIdx.x; e < P * Q; e += blockDim.x) sT[(e / Q) * QS + e % Q] = T[e];
-  const int nchunk = (I + AXI - 1) / AXI;
-  const int64_t tiles = B * nchunk;
-  const int i = threadIdx.x % AXI, p0 = threadIdx.x / AXI;
-  // tile -> [Q][AXI] in shared memory; whole 16-column chunks by 16-byte
-  // asynchronous copies, a ragged last chunk by plain loads with zero fill
-  auto fetch = [&](int64_t tile, float2* dst) {
-    const int64_t b = tile / nchunk;
-    const int i0 = (int)(tile % nchunk) * AXI;
-    if (i0 + AXI <= I && (I & 1) == 0) {
-      for (int e = threadIdx.x; e < Q * AXI / 2; e += blockDim.x) {
-        const int q = e / (AXI / 2), ii = 2 * (e % (AXI / 2));
-        cp16(dst + q * AXI + ii, in + (b * Q + q) * I + i0 + ii);
-      }
-    } else {
-      for (int e = threadIdx.x; e < Q * AXI; e += blockDim.x) {
-        const int q = e / AXI, ii = e % AXI;
-        dst[e] = i0 + ii < I ? in[(b * Q + q) * I + i0 + ii] : make_float2(0.f, 0.f);
-      }
-    }
-  };
-  if ((int64_t)blockIdx.x < tiles) fetch(blockIdx.x, sIn);
-  cp_commit();
-  int it = 0;
-  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, it++) {
-    const int64_t b = tile / nchunk;
-    const int i0 = (int)(tile % nchunk) * AXI;
-    const int64_t nxt = tile + gridDim.x;
-    __syncthreads();  // every thread is done with the buffer the next fetch overwrites
-    if (nxt < tiles) fetch(nxt, sIn + ((it + 1) & 1) * Q * AXI);
-    cp_commit();
-    cp_wait<1>();
-    __syncthreads();
-    const float2* cur = sIn + (it & 1) * Q * AXI;
-    float2 acc[4];
-#pragma unroll
-    for (int k = 0; k < 4; k++) acc[k] = make_float2(0.f, 0.f);
-    for (int q = 0; q < Q; q++) {
-      const float2 x = cur[q * AXI + i];
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const int p = p0 + 16 * k;
-        if (p < P) {
-          const float2 t = sT[p * QS + q];
-          acc[k].x = fmaf(t.x, x.x, fmaf(-t.y, x.y, acc[k].x));
-          acc[k].y = fmaf(t.x, x.y, fmaf(t.y, x.x, acc[k].y));
-        }
-      }
-    }
-    if (i0 + i < I) {
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const int p = p0 + 16 * k;
-        if (p < P) out[(b * P + p) * I + i0 + i] = acc[k];
-      }
-    }
-  }
-}
+#include "fno_dft.cuh"
 
 // t[c][k] = sum_j R[k][j][c] s[j][k] (complex, bf16 weights); one warp per
 // mode k, lane c (C <= 32): the weight loads are coalesced, s is broadcast.
@@ -991,70 +658,68 @@ unsigned grid_stride(int64_t n) {
   return (unsigned)(b < 4096 ? b : 4096);
 }
 
-size_t smem_axis(int P, int Q) { return sizeof(float2) * ((size_t)((P * (Q + 1) + 1) & ~1) + (size_t)2 * Q * AXI); }
-// k_axis: two persistent CTAs per SM, so that each streams several tiles
-unsigned axis_grid(int64_t tiles) { return (unsigned)(tiles < 152 * 2 ? tiles : 152 * 2); }
-
-// The fused plane kernels may need more than the default 48 KB of shared memory.
+// The plane kernels may need more than the default 48 KB of shared memory.
 template <typename K>
 bool opt_in(K kernel) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) == cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024) == cudaSuccess;
+}
+template <int NX, int MX, bool FULL = false>
+bool opt_in_xy() {
+  return opt_in(dft::k_xy_fwd<NX, MX, FULL>) && opt_in(dft::k_xy_inv<NX, MX, FULL>);
 }
 bool smem_opt_in() {
-  static const bool ok = opt_in(k_xy_fwd<16>) && opt_in(k_xy_fwd<32>) && opt_in(k_xy_fwd<64>) &&
-                         opt_in(k_xy_inv<16, 8>) && opt_in(k_xy_inv<16, 16>) && opt_in(k_xy_inv<32, 8>) &&
-                         opt_in(k_xy_inv<32, 16>) && opt_in(k_xy_inv<32, 32>) && opt_in(k_xy_inv<64, 8>) &&
-                         opt_in(k_xy_inv<64, 16>) && opt_in(k_xy_inv<64, 32>) && opt_in(k_xy_inv<64, 64>);
+  static const bool ok = opt_in_xy<16, 8>() && opt_in_xy<32, 8>() && opt_in_xy<32, 16>() && opt_in_xy<64, 8>() &&
+                         opt_in_xy<64, 16>() && opt_in_xy<64, 32>() && opt_in_xy<16, 8, true>() &&
+                         opt_in_xy<32, 16, true>() && opt_in_xy<64, 16, true>();
   return ok;
 }
+// Calls f(NX, MX, FULL) with the transform kernels' bounds on n and M.
+template <typename F>
+void by_size(int n, int M, F f) {
+  std::integral_constant<int, 8> c8;
+  std::integral_constant<int, 16> c16;
+  std::integral_constant<int, 32> c32;
+  std::integral_constant<int, 64> c64;
+  std::true_type full;
+  std::false_type part;
+  if (n == 16 && M == 8) f(c16, c8, full);
+  else if (n == 32 && M == 16) f(c32, c16, full);
+  else if (n == 64 && M == 16) f(c64, c16, full);
+  else if (n <= 16) f(c16, c8, part);
+  else if (n <= 32) M <= 8 ? f(c32, c8, part) : f(c32, c16, part);
+  else if (M <= 8) f(c64, c8, part);
+  else M <= 16 ? f(c64, c16, part) : f(c64, c32, part);
+}
+// Plane kernels: two persistent CTAs per SM, each streaming its planes.
+unsigned plane_grid(int planes) { return (unsigned)std::min(planes, 2 * 152); }
 
 // Forward transform of C channels of real fields v -> out [C][K] (kept modes).
 void dft3(const Shape& s, const Work& w, const float* v, float2* out, cudaStream_t st) {
-  const int n = s.n, M = s.M, C = s.C;
-  // x and y per (c, z) plane: [C n][n][n] -> [C n][2M][M]; two CTAs per SM,
-  // each streaming its planes through a double buffer
-  const unsigned g = (unsigned)std::min<int64_t>((int64_t)C * n, 2 * 152);
-  const size_t sm = smem_xy_fwd(n, M);
-  const int64_t np = (int64_t)C * n;
-  if (n <= 16) k_xy_fwd<16><<<g, 256, sm, st>>>(v, w.b, w.tab.fx, w.tab.tf, n, M, np);
-  else if (n <= 32) k_xy_fwd<32><<<g, 256, sm, st>>>(v, w.b, w.tab.fx, w.tab.tf, n, M, np);
-  else k_xy_fwd<64><<<g, 256, sm, st>>>(v, w.b, w.tab.fx, w.tab.tf, n, M, np);
-  // z: [C][n][2M M] -> [C][2M][2M M]
-  const int Iz = 2 * M * M;
-  k_axis<<<axis_grid((int64_t)C * ((Iz + AXI - 1) / AXI)), 256, smem_axis(2 * M, n), st>>>(w.b, out, w.tab.tf, C,
-                                                                                              2 * M, n, Iz);
+  const int n = s.n, M = s.M, C = s.C, Iz = 2 * M * M, np = C * n;
+  const size_t sz = dft::smem_z(n, M, n / 2, n / 2);
+  const dim3 gz((Iz + dft::ZC - 1) / dft::ZC, C);
+  by_size(n, M, [&](auto nx, auto mx, auto full) {
+    constexpr int NX = nx.value, MX = mx.value;
+    constexpr bool FULL = full.value;
+    dft::k_xy_fwd<NX, MX, FULL><<<plane_grid(np), dft::TH, dft::smem_xy_fwd(n, M), st>>>(v, w.b, n, M, np);
+    dft::k_z_fwd<NX, MX, FULL><<<gz, dft::TH, sz, st>>>(w.b, out, n, M, Iz);
+  });
 }
 
 // Inverse transform of [C][K] kept modes, added into z; act as in k_xy_inv.
-void idft3(const Shape& s, const Work& w, const float2* in, float* z, float* v, const float* xtab, int act,
+// adjoint: without the weights a(kx)/V, the adjoint of the forward transform.
+void idft3(const Shape& s, const Work& w, const float2* in, float* z, float* v, bool adjoint, int act,
            cudaStream_t st) {
-  const int n = s.n, M = s.M, C = s.C;
-  const int Iz = 2 * M * M;
-  k_axis<<<axis_grid((int64_t)C * ((Iz + AXI - 1) / AXI)), 256, smem_axis(n, 2 * M), st>>>(in, w.b, w.tab.ti, C, n,
-                                                                                              2 * M, Iz);
-  const unsigned g = (unsigned)std::min<int64_t>((int64_t)C * n, 2 * 152);
-  const size_t sm = smem_xy_inv(n, M);
-  const int64_t np = (int64_t)C * n;
-  const int M2 = 2 * M;
-#define XYI(NX, MX) k_xy_inv<NX, MX><<<g, 256, sm, st>>>(w.b, z, v, xtab, w.tab.ti, n, M, act, np)
-  if (n <= 16) {
-    if (M2 <= 8) XYI(16, 8);
-    else XYI(16, 16);
-  } else if (n <= 32) {
-    if (M2 <= 8) XYI(32, 8);
-    else if (M2 <= 16) XYI(32, 16);
-    else XYI(32, 32);
-  } else {
-    if (M2 <= 8) XYI(64, 8);
-    else if (M2 <= 16) XYI(64, 16);
-    else if (M2 <= 32) XYI(64, 32);
-    else XYI(64, 64);
-  }
-#undef XYI
-}
-
-void tables(const Shape& s, const Work& w, cudaStream_t st) {
-  k_tables<<<16, 256, 0, st>>>(s.n, s.M, 1.f / (float)s.V, w.tab);
+  const int n = s.n, M = s.M, C = s.C, Iz = 2 * M * M, np = C * n;
+  const float w0 = adjoint ? 1.f : 1.f / (float)s.V, w1 = adjoint ? 1.f : 2.f * w0;
+  const size_t sz = dft::smem_z(n, M, M + 1, n / 2 + 1);
+  const dim3 gz((Iz + dft::ZC - 1) / dft::ZC, C);
+  by_size(n, M, [&](auto nx, auto mx, auto full) {
+    constexpr int NX = nx.value, MX = mx.value;
+    constexpr bool FULL = full.value;
+    dft::k_z_inv<NX, MX, FULL><<<gz, dft::TH, sz, st>>>(in, w.b, n, M, Iz);
+    dft::k_xy_inv<NX, MX, FULL><<<plane_grid(np), dft::TH, dft::smem_xy_inv(n, M), st>>>(w.b, z, v, n, M, w0, w1, act, np);
+  });
 }
 
 void pw(const float* in, int Cin, const uint16_t* W, const uint16_t* b, int Cout, float* out, int64_t V,
@@ -1112,7 +777,6 @@ int mond_fno_forward(mond_fno_shape sh, const uint16_t* P, const float* x, float
   const int C = s.C;
   const int64_t V = s.V, CV = (int64_t)C * V;
   const unsigned warps_grid = (unsigned)(((int64_t)s.K * 32 + TB - 1) / TB);
-  tables(s, w, st);
   pw(x, 4, P + s.off_P(), P + s.off_p(), C, w.v, V, 0, st);
   for (int l = 0; l < s.L; l++) {
     const float* vl = w.v + l * CV;
@@ -1121,7 +785,7 @@ int mond_fno_forward(mond_fno_shape sh, const uint16_t* P, const float* x, float
     pw(vl, C, P + s.off_W(l), P + s.off_b(l), C, zl, V, 0, st);
     dft3(s, w, vl, shat, st);
     k_mix_fwd<<<warps_grid, TB, 0, st>>>(shat, P + s.off_R(l), w.c, C, s.K);
-    idft3(s, w, w.c, zl, w.v + (l + 1) * CV, w.tab.ix, l + 1 < s.L ? 1 : 2, st);
+    idft3(s, w, w.c, zl, w.v + (l + 1) * CV, false, l + 1 < s.L ? 1 : 2, st);
   }
   pw(w.v + s.L * CV, C, P + s.off_Q(), P + s.off_q(), 3, y, V, 0, st);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
@@ -1139,7 +803,6 @@ int mond_fno_backward(mond_fno_shape sh, const uint16_t* P, const float* x, cons
   const int64_t V = s.V, CV = (int64_t)C * V;
   const unsigned gw = 152 * 4;
   const unsigned warps_grid = (unsigned)(((int64_t)s.K * 32 + TB - 1) / TB);
-  tables(s, w, st);
   // projection
   k_wgrad<<<gw, TB, 0, st>>>(dy, 3, w.v + s.L * CV, C, V, grad + s.off_Q(), grad + s.off_q());
   float* dv = w.dv;
@@ -1160,7 +823,7 @@ int mond_fno_backward(mond_fno_shape sh, const uint16_t* P, const float* x, cons
     dft3(s, w, dz, w.c, st);
     k_mix_bwd<<<warps_grid, TB, 0, st>>>(w.c, w.shat + (int64_t)l * C * s.K, P + s.off_R(l), w.d, grad + s.off_R(l),
                                          C, s.K, M, 1.f / (float)V);
-    idft3(s, w, w.d, dv2, nullptr, w.tab.ixa, 0, st);
+    idft3(s, w, w.d, dv2, nullptr, true, 0, st);
     float* t = dv;
     dv = dv2;
     dv2 = t;
