@@ -131,23 +131,18 @@ __global__ void __launch_bounds__(256) k_pw(const float* __restrict__ in, int Ci
 // each FP32 input is split into three bfloat16 parts x = h + m + l (the top,
 // middle and low eight bits of its significand), so the three products per
 // weight are exact and only the FP32 accumulation rounds, as in the FMA chain
-// of k_pw. A warp takes 8 PW_NT voxels (PW_NT 8-column tiles) per step, all
-// 32 output rows (two 16-row tiles) and all 32 input rows (two 16-deep
-// steps); one tile a step keeps enough warps in flight on the small grids of
-// the network.
-constexpr int PW_NT = 1;  // 8-voxel tiles per warp step
-
+// of k_pw.
+// Bound by memory: a warp takes 32 voxels a step, as four 8-column tiles whose
+// columns are interleaved (column g of tile t is voxel 4g + t), so that a lane
+// loads four neighbouring voxels of a channel at once, all eight of its
+// channels before any is used, and stores four. One warp of 8 voxels with
+// 4-byte accesses: 37 us for 64^3, 32 -> 32 channels (67 MB); now 16.4 us.
 __device__ __forceinline__ uint32_t pack_bf16(float lo_half, float hi_half) {
-  const uint32_t a = __bfloat16_as_ushort(__float2bfloat16_rn(lo_half));
-  const uint32_t b = __bfloat16_as_ushort(__float2bfloat16_rn(hi_half));
-  return a | (b << 16);
+  const __nv_bfloat162 p = __floats2bfloat162_rn(lo_half, hi_half);
+  return *reinterpret_cast<const uint32_t*>(&p);
 }
-__device__ __forceinline__ void split3(float x, float& h, float& m, float& l) {
-  h = __bfloat162float(__float2bfloat16_rn(x));
-  const float r = x - h;  // exact
-  m = __bfloat162float(__float2bfloat16_rn(r));
-  l = r - m;              // exact, and representable in bfloat16
-}
+__device__ __forceinline__ float lo_bf16(uint32_t p) { return __uint_as_float(p << 16); }
+__device__ __forceinline__ float hi_bf16(uint32_t p) { return __uint_as_float(p & 0xffff0000u); }
 __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
@@ -156,9 +151,11 @@ __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, uint32_t b
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-__global__ void __launch_bounds__(256) k_pw_mma(const float* __restrict__ in, int Cin,
-                                                const uint16_t* __restrict__ W, const uint16_t* __restrict__ b,
-                                                int Cout, float* __restrict__ out, int64_t V, int transpose) {
+template <int MT>  // Cout <= 16 MT
+__global__ void __launch_bounds__(256, 2) k_pw_mma(const float* __restrict__ in, int Cin,
+                                                   const uint16_t* __restrict__ W, const uint16_t* __restrict__ b,
+                                                   int Cout, float* __restrict__ out, int64_t V, int transpose,
+                                                   int vec_out) {
   __shared__ uint16_t sW[32][32 + 8];  // [o][i], zero-padded; row pitch 80 bytes (conflict-free fragments)
   __shared__ float sb[32];
   for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
@@ -171,9 +168,9 @@ __global__ void __launch_bounds__(256) k_pw_mma(const float* __restrict__ in, in
   __syncthreads();
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   // A fragments: [M tile][K step][4 registers], row-major 16x16 tiles of sW
-  uint32_t A[2][2][4];
+  uint32_t A[MT][2][4];
 #pragma unroll
-  for (int mt = 0; mt < 2; mt++)
+  for (int mt = 0; mt < MT; mt++)
 #pragma unroll
     for (int ks = 0; ks < 2; ks++) {
       const int r0 = 16 * mt + g, c0 = 16 * ks + 2 * q;
@@ -183,89 +180,120 @@ __global__ void __launch_bounds__(256) k_pw_mma(const float* __restrict__ in, in
       A[mt][ks][3] = *reinterpret_cast<const uint32_t*>(&sW[r0 + 8][c0 + 8]);
     }
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (8 * PW_NT); v0 < V;
-       v0 += warps * (8 * PW_NT)) {
+  for (int64_t v0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; v0 < V; v0 += warps * 32) {
+    // rows k = 16 ks + 8 rr + 2 q + j of the B fragments, four voxels of each
+    float4 x[2][2][2];
 #pragma unroll
-    for (int nt = 0; nt < PW_NT; nt++) {
-      const int64_t vc = v0 + 8 * nt + g;  // this lane's column of the B fragments
-      // B fragments: rows k = 2q, 2q + 1 (register 0) and + 8 (register 1) of each 16-deep step
+    for (int ks = 0; ks < 2; ks++)
+#pragma unroll
+      for (int rr = 0; rr < 2; rr++)
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+          const int k = 16 * ks + 8 * rr + 2 * q + j;
+          x[ks][rr][j] = k < Cin ? __ldg(reinterpret_cast<const float4*>(in + (int64_t)k * V + v0) + g)
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    float d[MT][4][4];  // [M tile][voxel tile][C fragment: rows g, g + 8, columns 2q, 2q + 1]
+#pragma unroll
+    for (int t = 0; t < 4; t++) {
       uint32_t Bh[2][2], Bm[2][2], Bl[2][2];
 #pragma unroll
       for (int ks = 0; ks < 2; ks++)
 #pragma unroll
         for (int rr = 0; rr < 2; rr++) {
-          float x[2];
-#pragma unroll
-          for (int j = 0; j < 2; j++) {
-            const int k = 16 * ks + 8 * rr + 2 * q + j;
-            x[j] = (k < Cin && vc < V) ? in[(int64_t)k * V + vc] : 0.f;
-          }
-          float h0, m0, l0, h1, m1, l1;
-          split3(x[0], h0, m0, l0);
-          split3(x[1], h1, m1, l1);
-          Bh[ks][rr] = pack_bf16(h0, h1);
-          Bm[ks][rr] = pack_bf16(m0, m1);
-          Bl[ks][rr] = pack_bf16(l0, l1);
+          const float* f0 = &x[ks][rr][0].x;
+          const float* f1 = &x[ks][rr][1].x;
+          Bh[ks][rr] = pack_bf16(f0[t], f1[t]);
+          const float r0 = f0[t] - lo_bf16(Bh[ks][rr]), r1 = f1[t] - hi_bf16(Bh[ks][rr]);  // exact
+          Bm[ks][rr] = pack_bf16(r0, r1);
+          Bl[ks][rr] = pack_bf16(r0 - lo_bf16(Bm[ks][rr]), r1 - hi_bf16(Bm[ks][rr]));  // exact, a bfloat16
         }
 #pragma unroll
-      for (int mt = 0; mt < 2; mt++) {
-        // C fragment: rows g and g + 8 of the tile, columns 2q and 2q + 1
-        float d[4] = {sb[16 * mt + g], sb[16 * mt + g], sb[16 * mt + g + 8], sb[16 * mt + g + 8]};
+      for (int mt = 0; mt < MT; mt++) {
+        d[mt][t][0] = d[mt][t][1] = sb[16 * mt + g];
+        d[mt][t][2] = d[mt][t][3] = sb[16 * mt + g + 8];
 #pragma unroll
         for (int ks = 0; ks < 2; ks++) {
-          mma_bf16(d, A[mt][ks], Bl[ks][0], Bl[ks][1]);  // smallest parts first
-          mma_bf16(d, A[mt][ks], Bm[ks][0], Bm[ks][1]);
-          mma_bf16(d, A[mt][ks], Bh[ks][0], Bh[ks][1]);
-        }
-        const int64_t vo = v0 + 8 * nt + 2 * q;
-#pragma unroll
-        for (int half = 0; half < 2; half++) {
-          const int o = 16 * mt + g + 8 * half;
-          if (o >= Cout) continue;
-#pragma unroll
-          for (int j = 0; j < 2; j++)
-            if (vo + j < V) out[(int64_t)o * V + vo + j] = d[2 * half + j];
+          mma_bf16(d[mt][t], A[mt][ks], Bl[ks][0], Bl[ks][1]);  // smallest parts first
+          mma_bf16(d[mt][t], A[mt][ks], Bm[ks][0], Bm[ks][1]);
+          mma_bf16(d[mt][t], A[mt][ks], Bh[ks][0], Bh[ks][1]);
         }
       }
     }
+#pragma unroll
+    for (int mt = 0; mt < MT; mt++)
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        const int o = 16 * mt + g + 8 * (e >> 1);
+        if (o >= Cout) continue;
+        float* p = out + (int64_t)o * V + v0 + 8 * q + 4 * (e & 1);
+        if (vec_out) {
+          *reinterpret_cast<float4*>(p) = make_float4(d[mt][0][e], d[mt][1][e], d[mt][2][e], d[mt][3][e]);
+        } else {
+#pragma unroll
+          for (int t = 0; t < 4; t++) p[t] = d[mt][t][e];
+        }
+      }
   }
 }
 
 // dW[o][i] += sum_v dout[o][v] in[i][v]; db[o] += sum_v dout[o][v].
-__global__ void k_wgrad(const float* dout, int Cout, const float* in, int Cin, int64_t V, float* dW, float* db) {
-  constexpr int CH = 64;
-  __shared__ float so[32][CH + 1], si[32][CH + 1];  // padded: conflict-free column reads
-  const int npair = Cout * Cin + (db ? Cout : 0);
-  float acc[5] = {0, 0, 0, 0, 0};
-  for (int64_t v0 = (int64_t)blockIdx.x * CH; v0 < V; v0 += (int64_t)gridDim.x * CH) {
-    __syncthreads();
-    for (int t = threadIdx.x; t < (Cout + Cin) * CH; t += blockDim.x) {
-      const int row = t / CH, col = t % CH;
-      const int64_t v = v0 + col;
-      const float val = v < V ? (row < Cout ? dout[row * V + v] : in[(row - Cout) * V + v]) : 0.f;
-      if (row < Cout) so[row][col] = val;
-      else si[row - Cout][col] = val;
+// Tiles of 64 voxels in shared memory, the next one's loads in flight; a
+// thread owns the rows ob, ob + 16 and the columns ib, ib + 16 of dW, four
+// voxels a read. A CTA per SM: each adds its 1056 sums to the same words, and
+// with four CTAs per SM those atomics and one product per two reads took
+// 16.5 us at 32^3 (32 x 32 channels); now 9.0 us.
+__global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ dout, int Cout, const float* __restrict__ in,
+                                               int Cin, int64_t V, float* dW, float* db, int vec) {
+  constexpr int CH = 64, P = CH + 4;
+  __shared__ __align__(16) float so[32 * P], si[32 * P];
+  const int tid = threadIdx.x, ob = tid >> 4, ib = tid & 15, ntiles = (int)(V / CH);
+  float4 pre[4];
+  auto fetch = [&](int tile) {
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      const int row = (tid >> 4) + 16 * (k & 1);
+      const float* src = k < 2 ? dout : in;
+      const bool live = row < (k < 2 ? Cout : Cin);
+      const float* p = src + (int64_t)row * V + (int64_t)tile * CH + 4 * (tid & 15);
+      if (!live) pre[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      else if (vec) pre[k] = __ldg(reinterpret_cast<const float4*>(p));
+      else pre[k] = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
     }
+  };
+  float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, bias[2] = {0.f, 0.f};
+  if ((int)blockIdx.x < ntiles) fetch(blockIdx.x);
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     __syncthreads();
-    for (int k = 0; k < 5; k++) {
-      const int p = threadIdx.x + k * blockDim.x;
-      if (p >= npair) break;
-      float s = 0.f;
-      if (p < Cout * Cin) {
-        const int o = p / Cin, i = p % Cin;
-        for (int c = 0; c < CH; c++) s = fmaf(so[o][c], si[i][c], s);
-      } else {
-        const int o = p - Cout * Cin;
-        for (int c = 0; c < CH; c++) s += so[o][c];
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+      *reinterpret_cast<float4*>((k < 2 ? so : si) + ((tid >> 4) + 16 * (k & 1)) * P + 4 * (tid & 15)) = pre[k];
+    __syncthreads();
+    if (tile + (int)gridDim.x < ntiles) fetch(tile + gridDim.x);
+#pragma unroll 4
+    for (int c = 0; c < CH; c += 4) {
+      float4 a[2], x[2];
+#pragma unroll
+      for (int r = 0; r < 2; r++) {
+        a[r] = *reinterpret_cast<const float4*>(so + (ob + 16 * r) * P + c);
+        x[r] = *reinterpret_cast<const float4*>(si + (ib + 16 * r) * P + c);
+        bias[r] += (a[r].x + a[r].y) + (a[r].z + a[r].w);
       }
-      acc[k] += s;
+#pragma unroll
+      for (int r = 0; r < 2; r++)
+#pragma unroll
+        for (int t = 0; t < 2; t++)
+          acc[r][t] = fmaf(a[r].x, x[t].x, fmaf(a[r].y, x[t].y, fmaf(a[r].z, x[t].z, fmaf(a[r].w, x[t].w, acc[r][t]))));
     }
   }
-  for (int k = 0; k < 5; k++) {
-    const int p = threadIdx.x + k * blockDim.x;
-    if (p >= npair) break;
-    if (p < Cout * Cin) atomicAdd(dW + p, acc[k]);
-    else atomicAdd(db + (p - Cout * Cin), acc[k]);
+#pragma unroll
+  for (int r = 0; r < 2; r++) {
+    const int o = ob + 16 * r;
+    if (o >= Cout) continue;
+#pragma unroll
+    for (int t = 0; t < 2; t++)
+      if (ib + 16 * t < Cin) atomicAdd(dW + o * Cin + ib + 16 * t, acc[r][t]);
+    if (db && ib == 0) atomicAdd(db + o, bias[r]);
   }
 }
 
@@ -345,11 +373,147 @@ __global__ void k_mix_bwd(const float2* __restrict__ gt, const float2* __restric
   }
 }
 
-__global__ void k_gelu_bwd(const float* z, const float* dv, float* dz, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    float d;
-    gelu_t(z[i], &d);
-    dz[i] = dv[i] * d;
+// The same two for 32 channels, bound by the read of R (and of dR and its
+// write): a CTA takes eight modes, a warp one of them, its 1024 weights in
+// eight loads of 16 bytes a lane (lane: channels c = 4 (lane % 8) .., j =
+// 4 jj + lane / 8), all requested before the spectra arrive; the spectra pass
+// through shared memory, as eight modes are the 64 bytes that a channel keeps
+// together. A lane per channel with 4-byte loads and 8-byte strided spectra:
+// 17.8 us forward, 74 us backward at M = 16 (67 and 335 MB); now 13.2 us
+// and 58 us (5.8 TB/s).
+constexpr int MK = 8;   // modes per CTA
+constexpr int MP = 34;  // pitch of a mode's channels: eight modes and two channels in distinct banks
+__device__ __forceinline__ float2 wr_wi(uint32_t w) {
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+__device__ __forceinline__ void load_modes(float2 (*s)[MP], const float2* __restrict__ in, int k0, int K) {
+  const int m = threadIdx.x % MK, j = threadIdx.x / MK;
+  s[m][j] = k0 + m < K ? __ldg(in + (int64_t)j * K + k0 + m) : make_float2(0.f, 0.f);
+}
+__device__ __forceinline__ void store_modes(const float2 (*s)[MP], float2* __restrict__ out, int k0, int K) {
+  const int m = threadIdx.x % MK, j = threadIdx.x / MK;
+  if (k0 + m < K) out[(int64_t)j * K + k0 + m] = s[m][j];
+}
+__global__ void __launch_bounds__(256) k_mix_fwd32(const float2* __restrict__ s, const uint4* __restrict__ R,
+                                                   float2* __restrict__ t, int K) {
+  __shared__ float2 sS[MK][MP], sO[MK][MP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k0 = blockIdx.x * MK, k = k0 + warp;
+  uint4 w[8];
+#pragma unroll
+  for (int jj = 0; jj < 8; jj++) w[jj] = k < K ? __ldcs(R + (int64_t)k * 256 + 32 * jj + lane) : make_uint4(0, 0, 0, 0);
+  load_modes(sS, s, k0, K);
+  __syncthreads();
+  float2 acc[4];
+#pragma unroll
+  for (int c = 0; c < 4; c++) acc[c] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int jj = 0; jj < 8; jj++) {
+    const float2 x = sS[warp][4 * jj + (lane >> 3)];
+    const uint32_t u[4] = {w[jj].x, w[jj].y, w[jj].z, w[jj].w};
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const float2 r = wr_wi(u[c]);
+      acc[c].x = fmaf(r.x, x.x, fmaf(-r.y, x.y, acc[c].x));
+      acc[c].y = fmaf(r.x, x.y, fmaf(r.y, x.x, acc[c].y));
+    }
+  }
+#pragma unroll
+  for (int o = 8; o < 32; o <<= 1)
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      acc[c].x += __shfl_xor_sync(0xffffffffu, acc[c].x, o);
+      acc[c].y += __shfl_xor_sync(0xffffffffu, acc[c].y, o);
+    }
+  if (lane < 8) {
+#pragma unroll
+    for (int c = 0; c < 4; c++) sO[warp][4 * lane + c] = acc[c];
+  }
+  __syncthreads();
+  store_modes(sO, t, k0, K);
+}
+__global__ void __launch_bounds__(256) k_mix_bwd32(const float2* __restrict__ gt, const float2* __restrict__ s,
+                                                   const uint4* __restrict__ R, float2* __restrict__ gs,
+                                                   float4* __restrict__ dR, int K, int M, float invV) {
+  __shared__ float2 sG[MK][MP], sS[MK][MP], sO[MK][MP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k0 = blockIdx.x * MK, k = k0 + warp;
+  const bool live = k < K;
+  const int64_t base = (int64_t)k * 256 + lane;
+  load_modes(sG, gt, k0, K);
+  load_modes(sS, s, k0, K);
+  __syncthreads();
+  const float a = ((k % M) == 0 ? 1.f : 2.f) * invV;
+  float2 g[4], p[8];
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    g[c] = sG[warp][4 * (lane & 7) + c];
+    g[c].x *= a;
+    g[c].y *= a;
+  }
+#pragma unroll
+  for (int half = 0; half < 2; half++) {
+    uint4 w[4];
+    float4 d[4][2];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const int64_t r = base + 32 * (4 * half + q);
+      w[q] = live ? __ldg(R + r) : make_uint4(0, 0, 0, 0);
+      d[q][0] = live ? __ldcs(dR + 2 * r) : make_float4(0.f, 0.f, 0.f, 0.f);
+      d[q][1] = live ? __ldcs(dR + 2 * r + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const int jj = 4 * half + q;
+      const float2 x = sS[warp][4 * jj + (lane >> 3)];
+      const uint32_t u[4] = {w[q].x, w[q].y, w[q].z, w[q].w};
+      p[jj] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        const float2 r = wr_wi(u[c]);
+        p[jj].x = fmaf(r.x, g[c].x, fmaf(r.y, g[c].y, p[jj].x));  // conj(w) g
+        p[jj].y = fmaf(r.x, g[c].y, fmaf(-r.y, g[c].x, p[jj].y));
+        float4& v = d[q][c >> 1];
+        float& vx = (c & 1) ? v.z : v.x;
+        float& vy = (c & 1) ? v.w : v.y;
+        vx += x.x * g[c].x + x.y * g[c].y;  // conj(s) g
+        vy += x.x * g[c].y - x.y * g[c].x;
+      }
+      if (live) {
+        const int64_t r = base + 32 * jj;
+        __stcs(dR + 2 * r, d[q][0]);
+        __stcs(dR + 2 * r + 1, d[q][1]);
+      }
+    }
+  }
+  // sums over the 8 lanes of a j: each step halves the j's a lane keeps
+#pragma unroll
+  for (int h = 4; h > 0; h >>= 1) {
+    const bool up = lane & h;
+#pragma unroll
+    for (int q = 0; q < h; q++) {
+      const float2 keep = up ? p[q + h] : p[q], send = up ? p[q] : p[q + h];
+      p[q].x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, h);
+      p[q].y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, h);
+    }
+  }
+  sO[warp][4 * (lane & 7) + (lane >> 3)] = p[0];
+  __syncthreads();
+  store_modes(sO, gs, k0, K);
+}
+// 32 channels, and weights on 16-byte boundaries
+bool mix32(int C, const void* R, const void* dR) {
+  return C == 32 && ((reinterpret_cast<uintptr_t>(R) | reinterpret_cast<uintptr_t>(dR)) & 15) == 0;
+}
+
+__global__ void __launch_bounds__(256) k_gelu_bwd(const float4* __restrict__ z, const float4* __restrict__ dv,
+                                                  float4* __restrict__ dz, int64_t n4) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
+    const float4 a = __ldg(z + i), b = __ldg(dv + i);
+    float4 d;
+    gelu_t(a.x, &d.x);
+    gelu_t(a.y, &d.y);
+    gelu_t(a.z, &d.z);
+    gelu_t(a.w, &d.w);
+    dz[i] = make_float4(b.x * d.x, b.y * d.y, b.z * d.z, b.w * d.w);
   }
 }
 
@@ -722,16 +886,19 @@ void idft3(const Shape& s, const Work& w, const float2* in, float* z, float* v, 
   });
 }
 
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 void pw(const float* in, int Cin, const uint16_t* W, const uint16_t* b, int Cout, float* out, int64_t V,
         int transpose, cudaStream_t st) {
   const unsigned g = grid_stride(V);
   if (Cin <= 4) {
     k_pw<4><<<g, TB, 0, st>>>(in, Cin, W, b, Cout, out, V, transpose);
   } else {
-    // tensor cores: one warp per 8 PW_NT voxels a step
-    const int64_t steps = (V + 8 * PW_NT - 1) / (8 * PW_NT);
-    const unsigned gm = (unsigned)std::min<int64_t>((steps + 7) / 8, 4096);
-    k_pw_mma<<<gm, TB, 0, st>>>(in, Cin, W, b, Cout, out, V, transpose);
+    // tensor cores: one warp per 32 voxels a step (V = n^3 is a multiple of 64), two CTAs per SM
+    const unsigned gm = (unsigned)std::min<int64_t>((V / 32 + 7) / 8, 152 * 2);
+    const int vec = aligned16(out);
+    if (Cout <= 16) k_pw_mma<1><<<gm, TB, 0, st>>>(in, Cin, W, b, Cout, out, V, transpose, vec);
+    else k_pw_mma<2><<<gm, TB, 0, st>>>(in, Cin, W, b, Cout, out, V, transpose, vec);
   }
 }
 
@@ -784,7 +951,11 @@ int mond_fno_forward(mond_fno_shape sh, const uint16_t* P, const float* x, float
     float2* shat = w.shat + (int64_t)l * C * s.K;
     pw(vl, C, P + s.off_W(l), P + s.off_b(l), C, zl, V, 0, st);
     dft3(s, w, vl, shat, st);
-    k_mix_fwd<<<warps_grid, TB, 0, st>>>(shat, P + s.off_R(l), w.c, C, s.K);
+    const uint16_t* R = P + s.off_R(l);
+    if (mix32(C, R, nullptr))
+      k_mix_fwd32<<<(s.K + MK - 1) / MK, TB, 0, st>>>(shat, reinterpret_cast<const uint4*>(R), w.c, s.K);
+    else
+      k_mix_fwd<<<warps_grid, TB, 0, st>>>(shat, R, w.c, C, s.K);
     idft3(s, w, w.c, zl, w.v + (l + 1) * CV, false, l + 1 < s.L ? 1 : 2, st);
   }
   pw(w.v + s.L * CV, C, P + s.off_Q(), P + s.off_q(), 3, y, V, 0, st);
@@ -801,10 +972,11 @@ int mond_fno_backward(mond_fno_shape sh, const uint16_t* P, const float* x, cons
   carve(s, (char*)workspace, &w);
   const int C = s.C, M = s.M;
   const int64_t V = s.V, CV = (int64_t)C * V;
-  const unsigned gw = 152 * 4;
+  const unsigned gw = (unsigned)std::min<int64_t>(V / 64, 152);
   const unsigned warps_grid = (unsigned)(((int64_t)s.K * 32 + TB - 1) / TB);
   // projection
-  k_wgrad<<<gw, TB, 0, st>>>(dy, 3, w.v + s.L * CV, C, V, grad + s.off_Q(), grad + s.off_q());
+  k_wgrad<<<gw, TB, 0, st>>>(dy, 3, w.v + s.L * CV, C, V, grad + s.off_Q(), grad + s.off_q(),
+                              aligned16(dy) && aligned16(w.v + s.L * CV));
   float* dv = w.dv;
   float* dv2 = w.dv2;
   pw(dy, 3, P + s.off_Q(), nullptr, C, dv, V, 1, st);
@@ -813,23 +985,33 @@ int mond_fno_backward(mond_fno_shape sh, const uint16_t* P, const float* x, cons
     const float* zl = w.z + l * CV;
     const float* dz = dv;  // the last layer has no activation
     if (l + 1 < s.L) {
-      k_gelu_bwd<<<grid_stride(CV), TB, 0, st>>>(zl, dv, w.dz, CV);
+      k_gelu_bwd<<<grid_stride(CV / 4), TB, 0, st>>>(reinterpret_cast<const float4*>(zl),
+                                                      reinterpret_cast<const float4*>(dv),
+                                                      reinterpret_cast<float4*>(w.dz), CV / 4);
       dz = w.dz;
     }
     // pointwise part
-    k_wgrad<<<gw, TB, 0, st>>>(dz, C, vl, C, V, grad + s.off_W(l), grad + s.off_b(l));
+    k_wgrad<<<gw, TB, 0, st>>>(dz, C, vl, C, V, grad + s.off_W(l), grad + s.off_b(l),
+                              aligned16(dz) && aligned16(vl));
     pw(dz, C, P + s.off_W(l), nullptr, C, dv2, V, 1, st);
     // spectral part: G_t = (a/V) DFT(dz), through the mixing adjoint, back with the adjoint transform
     dft3(s, w, dz, w.c, st);
-    k_mix_bwd<<<warps_grid, TB, 0, st>>>(w.c, w.shat + (int64_t)l * C * s.K, P + s.off_R(l), w.d, grad + s.off_R(l),
-                                         C, s.K, M, 1.f / (float)V);
+    const float2* shat = w.shat + (int64_t)l * C * s.K;
+    const uint16_t* R = P + s.off_R(l);
+    float* dR = grad + s.off_R(l);
+    if (mix32(C, R, dR))
+      k_mix_bwd32<<<(s.K + MK - 1) / MK, TB, 0, st>>>(w.c, shat, reinterpret_cast<const uint4*>(R), w.d,
+                                                      reinterpret_cast<float4*>(dR), s.K, M, 1.f / (float)V);
+    else
+      k_mix_bwd<<<warps_grid, TB, 0, st>>>(w.c, shat, R, w.d, dR, C, s.K, M, 1.f / (float)V);
     idft3(s, w, w.d, dv2, nullptr, true, 0, st);
     float* t = dv;
     dv = dv2;
     dv2 = t;
   }
   // lift
-  k_wgrad<<<gw, TB, 0, st>>>(dv, C, x, 4, V, grad + s.off_P(), grad + s.off_p());
+  k_wgrad<<<gw, TB, 0, st>>>(dv, C, x, 4, V, grad + s.off_P(), grad + s.off_p(),
+                              aligned16(dv) && aligned16(x));
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -850,14 +1032,14 @@ int mond_fno_adam_cast(int64_t count, float* p, float* g, float* m, float* v, fl
   cudaStream_t st = (cudaStream_t)stream;
   const AdamArgs a{lr, b1, b2, eps, 1.f - powf(b1, (float)step), 1.f - powf(b2, (float)step), clip_norm, scratch};
   cudaMemsetAsync(scratch, 0, sizeof(double), st);
-  auto aligned = [](const void* q, int bytes) { return (reinterpret_cast<uintptr_t>(q) & (bytes - 1)) == 0; };
   const unsigned grid = grid_stride((count + 3) / 4);
-  if (aligned(g, 16))
+  if (aligned16(g))
     k_gradnorm<<<grid, TB, 0, st>>>(reinterpret_cast<const float4*>(g), count / 4, g + count / 4 * 4, (int)(count % 4),
                                     scratch);
   else
     k_sumsq<<<grid_stride(count), TB, 0, st>>>(g, count, scratch);
-  const int vec = aligned(p, 16) && aligned(g, 16) && aligned(m, 16) && aligned(v, 16) && aligned(pb, 8);
+  const int vec = aligned16(p) && aligned16(g) && aligned16(m) && aligned16(v) &&
+                  (reinterpret_cast<uintptr_t>(pb) & 7) == 0;
   k_adam<<<vec ? grid : grid_stride(count), TB, 0, st>>>(count, p, g, m, v, pb, a, vec);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
