@@ -527,7 +527,10 @@ __global__ void k_sumsq(const float* t, int64_t n, double* out) {
 
 __global__ void k_loss(const float* y, const float* t, float* dy, int64_t n, const double* tnorm, float weight,
                        double* loss) {
-  const double inv = 1.0 / fmax(*tnorm, 1e-300);
+  __shared__ double s_inv;
+  if (threadIdx.x == 0) s_inv = 1.0 / fmax(*tnorm, 1e-300);
+  __syncthreads();
+  const double inv = s_inv;
   double s = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float d = y[i] - t[i];
@@ -544,7 +547,7 @@ __global__ void k_loss(const float* y, const float* t, float* dy, int64_t n, con
 // rate. A thread whose values leave the range where that is exact enough
 // (past 1e18 in size, all below 1e-12, infinities, NaNs) sums them in FP64.
 // 134e6 floats: 252 us (FP64
-// sums) -> 96 us, 5.6 TB/s.
+// sums) -> 96 us, 5.6 TB/s; 786432 floats: 40 -> 6 us.
 __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, int64_t n4, const float* __restrict__ tail,
                                                   int ntail, double* out) {
   __shared__ double part[8];
@@ -569,8 +572,14 @@ __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, 
   double r = 0.0;
   const float sum = (s[0] + s[1]) + (s[2] + s[3]);
   if (isfinite(sum) && top < 1e18f && (top == 0.f || top > 1e-12f)) {
+    // the four sums as one float pair, then one FP64 addition a thread
 #pragma unroll
-    for (int k = 0; k < 4; k++) r += (double)s[k] + (double)c[k];
+    for (int k = 1; k < 4; k++) {
+      const float u = __fadd_rn(s[0], s[k]), d = __fsub_rn(u, s[0]);
+      c[0] += __fadd_rn(__fadd_rn(__fsub_rn(s[0], __fsub_rn(u, d)), __fsub_rn(s[k], d)), c[k]);
+      s[0] = u;
+    }
+    r = (double)s[0] + (double)c[0];
   } else {
     for (int64_t i = i0; i < n4; i += stride) {
       const float4 x = __ldg(t + i);
@@ -613,7 +622,10 @@ __device__ __forceinline__ void adam1(const AdamArgs& a, float scale, float& p, 
 // (two kernels) -> 0.68 ms, 6.7 TB/s.
 __global__ void __launch_bounds__(256) k_adam(int64_t n, float* p, float* g, float* m, float* v, uint16_t* pb,
                                               AdamArgs a, int vec) {
-  const float scale = adam_scale(a);
+  __shared__ float s_scale;  // one thread takes the FP64 square root
+  if (threadIdx.x == 0) s_scale = adam_scale(a);
+  __syncthreads();
+  const float scale = s_scale;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t n4 = vec ? n / 4 : 0;
 #pragma unroll 2
@@ -701,15 +713,75 @@ __global__ void k_coarsen(int N, int n, const float* __restrict__ fine, const fl
   }
 }
 
+// The same with 16-byte loads, rows split over the CTA (N / 4 lanes along x,
+// RY row groups), so that a thread has several loads in flight. Bound by the
+// read: 256^3 -> 64^3, three components (201 MB): 55 us with 4-byte loads, now
+// 49 us (4.1 TB/s).
+__global__ void __launch_bounds__(256, 6) k_coarsen4(int N, int n, const float4* __restrict__ fine,
+                                                  const float4* __restrict__ fine2, float* __restrict__ coarse,
+                                                  const float* __restrict__ scale) {
+  extern __shared__ __align__(16) float sx[];  // [RY][N]
+  const int f = N / n, TX = N / 4, RY = blockDim.y, xq = threadIdx.x, ry = threadIdx.y;
+  const int row = (blockIdx.z * n + blockIdx.y) * n + blockIdx.x;
+  const int y = blockIdx.x, z = blockIdx.y, c = blockIdx.z;
+  const int64_t base = (((int64_t)c * N + z * f) * N + y * f) * TX + xq;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  int off = ry * TX, dy = ry;  // row dy of plane dz: f N TX is below 2^31 / 64 (N <= 1024)
+  while (dy >= f) dy -= f, off += (N - f) * TX;
+#pragma unroll 4
+  for (int r = ry; r < f * f; r += RY) {
+    float4 v = __ldcs(fine + base + off);
+    if (fine2) {
+      const float4 u = __ldcs(fine2 + base + off);
+      v = make_float4(0.5f * (v.x + u.x), 0.5f * (v.y + u.y), 0.5f * (v.z + u.z), 0.5f * (v.w + u.w));
+    }
+    acc = make_float4(acc.x + v.x, acc.y + v.y, acc.z + v.z, acc.w + v.w);
+    dy += RY;
+    off += RY * TX;
+    while (dy >= f) dy -= f, off += (N - f) * TX;
+  }
+  const float d = (float)f * f * f * (scale ? *scale : 1.f);
+  if (f % 4 == 0) {  // a quad lies in one coarse cell
+    sx[ry * TX + xq] = (acc.x + acc.y) + (acc.z + acc.w);
+    __syncthreads();
+    for (int xc = ry * TX + xq; xc < n; xc += RY * TX) {
+      float a = 0.f;
+      for (int r = 0; r < RY; r++)
+        for (int t = 0; t < f / 4; t++) a += sx[r * TX + xc * (f / 4) + t];
+      coarse[(int64_t)row * n + xc] = a / d;
+    }
+    return;
+  }
+  *reinterpret_cast<float4*>(sx + ry * N + 4 * xq) = acc;
+  __syncthreads();
+  for (int xc = ry * TX + xq; xc < n; xc += RY * TX) {
+    float a = 0.f;
+    for (int r = 0; r < RY; r++)
+      for (int dx = 0; dx < f; dx++) a += sx[r * N + xc * f + dx];
+    coarse[(int64_t)row * n + xc] = a / d;
+  }
+}
+
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 void launch_coarsen(int N, int n, int ncomp, const float* fine, const float* fine2, float* coarse,
                     const float* scale, cudaStream_t st) {
+  if (N % 4 == 0 && N <= 1024 && ncomp < 65536 && aligned16(fine) && aligned16(fine2)) {
+    const int f = N / n, TX = N / 4, RY = std::min(f * f, 256 / TX);
+    k_coarsen4<<<dim3(n, n, ncomp), dim3(TX, RY), sizeof(float) * N * RY, st>>>(
+        N, n, reinterpret_cast<const float4*>(fine), reinterpret_cast<const float4*>(fine2), coarse, scale);
+    return;
+  }
   const int threads = N < 256 ? ((N + 31) / 32) * 32 : 256;
   k_coarsen<<<(unsigned)(ncomp * n * n), threads, sizeof(float) * N, st>>>(N, n, fine, fine2, coarse, scale);
 }
 
 __global__ void k_input(int n, float a0, const float* g, const double* sumsq, float* x, float* scale_out) {
   const int64_t V = (int64_t)n * n * n;
-  const float s = (float)sqrt(fmax(*sumsq / (3.0 * V), 1e-60));
+  __shared__ float s_rms;  // one thread a CTA does the FP64 arithmetic
+  if (threadIdx.x == 0) s_rms = (float)sqrt(fmax(*sumsq / (3.0 * V), 1e-60));
+  __syncthreads();
+  const float s = s_rms;
   if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = s;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
     const float gx = g[v], gy = g[V + v], gz = g[2 * V + v];
@@ -792,6 +864,91 @@ __global__ void k_up_axis(int n, int N, int64_t inner, int64_t chunk, const floa
   }
 }
 
+// All three axes in one pass, for factors f = N/n and coarse sides n that are
+// multiples of four: a CTA takes one coarse interval along y and UPZ of them
+// along z in turn (four of the f fine planes of each: blockIdx.z), interpolates
+// the coarse rows along y, then z (in shared memory, on the coarse x), and
+// writes 4 f fine rows, a thread always the same four neighbouring x. Bound by the write; the
+// three passes it replaces also wrote and read the two steps between: 64^3 ->
+// 256^3, three components (201 MB): 120 us, now 54 us
+// (3.8 TB/s; its instructions take 80% of the issue slots). Other factors and
+// sides keep the three passes.
+constexpr int UPZ = 4;
+size_t smem_up3(int n, int N) { return sizeof(float) * (16 * (size_t)n + 8 * (size_t)N + 4 * (size_t)(N / n)); }
+__global__ void __launch_bounds__(256) k_up3(int n, int N, const float4* __restrict__ in, float4* __restrict__ out,
+                                             const float* __restrict__ scale) {
+  extern __shared__ __align__(16) float sm[];
+  const int f = N / n, n4 = n / 4, TX = N / 4, RY = blockDim.y;  // TX float4s: a fine row, or f coarse rows
+  const int xq = threadIdx.x, ry = threadIdx.y, q = xq / n4, i4 = xq - q * n4;
+  float4* sC = reinterpret_cast<float4*>(sm);  // [4 z][4 y][n], coarse
+  float4* sP = sC + 16 * n4;                   // [4 z][f][n], fine along y
+  float4* sQ = sP + 4 * TX;                    // [4][f][n], fine along z too
+  float4* sw = sQ + 4 * TX;                    // [f] weights of the fine positions of an interval
+  const int jy = blockIdx.x, jz0 = UPZ * blockIdx.y, c = blockIdx.z % 3, q0 = 4 * (blockIdx.z / 3);
+  auto wrap = [](int i, int m) { return i < 0 ? i + m : i < m ? i : i - m; };
+  for (int p = ry * TX + xq; p < f; p += RY * TX) {
+    float w[4];
+    cubic_w((f / 2 + p + 0.5f) / f - 0.5f, w);  // f j + f/2 + p is that far past the coarse position j
+    sw[p] = make_float4(w[0], w[1], w[2], w[3]);
+  }
+  __syncthreads();
+  auto mix = [](float4 w, float4 a, float4 b, float4 d, float4 e, float s) {
+    return make_float4(s * (w.x * a.x + w.y * b.x + w.z * d.x + w.w * e.x),
+                       s * (w.x * a.y + w.y * b.y + w.z * d.y + w.w * e.y),
+                       s * (w.x * a.z + w.y * b.z + w.z * d.z + w.w * e.z),
+                       s * (w.x * a.w + w.y * b.w + w.z * d.w + w.w * e.w));
+  };
+  // x: weights and coarse cells of this thread's four positions X0 + k of the
+  // coarse cell i, which lie past the coarse position i - 1 or, from f/2 on, i
+  const float s = *scale;
+  const int X0 = 4 * xq, i = X0 / f, x0 = X0 - i * f, h = f / 2;
+  float4 wx[4];
+#pragma unroll
+  for (int k = 0; k < 4; k++) wx[k] = sw[x0 + k < h ? x0 + k + h : x0 + k - h];
+  const int first = i - (x0 < h ? 2 : 1);
+  const bool far = x0 < h && x0 + 2 >= h;  // the taps move on by a cell between X0 + 1 and X0 + 2 (h is even)
+  int idx[5];
+#pragma unroll
+  for (int k = 0; k < 5; k++) idx[k] = wrap(first + k, n);
+  const int Y0 = f * jy + h;
+  for (int step = 0; step < UPZ; step++) {
+    // coarse plane jz - 1 + k is in slot (step + k) % 4 of sC and sP
+    const int jz = jz0 + step, k0 = step ? 3 : 0;
+    for (int r = 4 * k0 + ry * f + q; r < 16; r += RY * f) {
+      const int z = wrap(jz - 1 + r / 4, n), y = wrap(jy - 1 + r % 4, n);
+      sC[(4 * ((step + r / 4) & 3) + r % 4) * n4 + i4] = __ldg(in + (((int64_t)c * n + z) * n + y) * n4 + i4);
+    }
+    __syncthreads();
+    for (int k = k0 + ry; k < 4; k += RY) {
+      const int slot = (step + k) & 3;
+      const float4* v = sC + 4 * slot * n4 + i4;
+      sP[slot * TX + xq] = mix(sw[q], v[0], v[n4], v[2 * n4], v[3 * n4], 1.f);
+    }
+    __syncthreads();
+    {
+      const float4 a = sP[(step & 3) * TX + xq], b = sP[((step + 1) & 3) * TX + xq],
+                   d = sP[((step + 2) & 3) * TX + xq], e = sP[((step + 3) & 3) * TX + xq];
+      for (int z = ry; z < 4; z += RY) sQ[z * TX + xq] = mix(sw[q0 + z], a, b, d, e, s);
+    }
+    __syncthreads();
+    const int Z0 = f * jz + h + q0;
+    int qz = 0, qy = ry;  // fine row: plane Z0 + qz, row Y0 + qy of the interval
+    for (;; qy += RY) {
+      while (qy >= f) qy -= f, qz++;
+      if (qz >= 4) break;
+      const float* v = reinterpret_cast<const float*>(sQ) + (qz * f + qy) * n;
+      const float a = v[idx[0]], b = v[idx[1]], d = v[idx[2]], e = v[idx[3]], g = v[idx[4]];
+      const float a2 = far ? b : a, b2 = far ? d : b, d2 = far ? e : d, e2 = far ? g : e;
+      float4 o;
+      o.x = wx[0].x * a + wx[0].y * b + wx[0].z * d + wx[0].w * e;
+      o.y = wx[1].x * a + wx[1].y * b + wx[1].z * d + wx[1].w * e;
+      o.z = wx[2].x * a2 + wx[2].y * b2 + wx[2].z * d2 + wx[2].w * e2;
+      o.w = wx[3].x * a2 + wx[3].y * b2 + wx[3].z * d2 + wx[3].w * e2;
+      __stcs(out + (((int64_t)c * N + wrap(Z0 + qz, N)) * N + wrap(Y0 + qy, N)) * TX + xq, o);
+    }
+  }
+}
+
 // Sphere mixture on the mesh (Plummer: 3M/(4 pi a^3) (1 + r^2/a^2)^{-5/2};
 // Hernquist: M a / (2 pi r (r + a)^3) with r >= 1/2 px), truncated at rmax.
 __global__ void k_mixture(int N, float s, int K, const float* centre, const float* mass, const float* radius,
@@ -820,6 +977,16 @@ __global__ void k_mixture(int N, float s, int K, const float* centre, const floa
 unsigned grid_stride(int64_t n) {
   int64_t b = (n + TB - 1) / TB;
   return (unsigned)(b < 4096 ? b : 4096);
+}
+
+// *out += the sum of the squares of t.
+void sumsq(const float* t, int64_t n, double* out, cudaStream_t st) {
+  if (aligned16(t))
+    // eight vectors a thread at least: a thread ends with FP64 sums
+    k_gradnorm<<<grid_stride((n + 31) / 32), TB, 0, st>>>(reinterpret_cast<const float4*>(t), n / 4, t + n / 4 * 4,
+                                                        (int)(n % 4), out);
+  else
+    k_sumsq<<<grid_stride(n), TB, 0, st>>>(t, n, out);
 }
 
 // The plane kernels may need more than the default 48 KB of shared memory.
@@ -885,8 +1052,6 @@ void idft3(const Shape& s, const Work& w, const float2* in, float* z, float* v, 
     dft::k_xy_inv<NX, MX, FULL><<<plane_grid(np), dft::TH, dft::smem_xy_inv(n, M), st>>>(w.b, z, v, n, M, w0, w1, act, np);
   });
 }
-
-bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 void pw(const float* in, int Cin, const uint16_t* W, const uint16_t* b, int Cout, float* out, int64_t V,
         int transpose, cudaStream_t st) {
@@ -1021,7 +1186,7 @@ int mond_fno_loss(int64_t count, const float* y, const float* t, float* dy, floa
   cudaStream_t st = (cudaStream_t)stream;
   double* tn = loss_acc + 1;  // scratch slot after the accumulator
   cudaMemsetAsync(tn, 0, sizeof(double), st);
-  k_sumsq<<<grid_stride(count), TB, 0, st>>>(t, count, tn);
+  sumsq(t, count, tn, st);
   k_loss<<<grid_stride(count), TB, 0, st>>>(y, t, dy, count, tn, weight, loss_acc);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
@@ -1033,11 +1198,7 @@ int mond_fno_adam_cast(int64_t count, float* p, float* g, float* m, float* v, fl
   const AdamArgs a{lr, b1, b2, eps, 1.f - powf(b1, (float)step), 1.f - powf(b2, (float)step), clip_norm, scratch};
   cudaMemsetAsync(scratch, 0, sizeof(double), st);
   const unsigned grid = grid_stride((count + 3) / 4);
-  if (aligned16(g))
-    k_gradnorm<<<grid, TB, 0, st>>>(reinterpret_cast<const float4*>(g), count / 4, g + count / 4 * 4, (int)(count % 4),
-                                    scratch);
-  else
-    k_sumsq<<<grid_stride(count), TB, 0, st>>>(g, count, scratch);
+  sumsq(g, count, scratch, st);
   const int vec = aligned16(p) && aligned16(g) && aligned16(m) && aligned16(v) &&
                   (reinterpret_cast<uintptr_t>(pb) & 7) == 0;
   k_adam<<<vec ? grid : grid_stride(count), TB, 0, st>>>(count, p, g, m, v, pb, a, vec);
@@ -1064,7 +1225,7 @@ int mond_fno_input(int N, int n, float a0, const float* gN, float* x, float* sca
   launch_coarsen(N, n, 3, gN, nullptr, x, nullptr, st);
   double* acc = reinterpret_cast<double*>(scale_out + 2);  // scale_out must have room for 2 + 2 floats
   cudaMemsetAsync(acc, 0, sizeof(double), st);
-  k_sumsq<<<grid_stride(3 * V), TB, 0, st>>>(x, 3 * V, acc);
+  sumsq(x, 3 * V, acc, st);
   k_input<<<grid_stride(V), TB, 0, st>>>(n, a0, x, acc, x, scale_out);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
@@ -1076,13 +1237,19 @@ size_t mond_fno_output_scratch_bytes(int N, int n) {
 
 int mond_fno_output(int N, int n, const float* y, const float* scale, float* H, void* scratch, void* stream) {
   if (!y || !scale || !H || !scratch || n <= 0 || N % n) return -1;
+  const int f = N / n;
+  if (f > 64) return -1;
   cudaStream_t st = (cudaStream_t)stream;
+  if (f % 4 == 0 && n % 4 == 0 && N <= 512 && aligned16(y) && aligned16(H)) {
+    k_up3<<<dim3(n, n / UPZ, 3 * (f / 4)), dim3(N / 4, 256 / (N / 4)), smem_up3(n, N), st>>>(
+        n, N, reinterpret_cast<const float4*>(y), reinterpret_cast<float4*>(H), scale);
+    return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  }
   float* t1 = (float*)scratch;              // [3 n n][N]   x upsampled
   float* t2 = t1 + (size_t)3 * n * n * N;   // [3 n][N][N]  x, y upsampled
   const int threads = N < 256 ? ((N + 31) / 32) * 32 : 256;
   k_up_x<<<(unsigned)(3 * n * n), threads, 0, st>>>(n, N, y, t1);
-  if (N / n > 64) return -1;
-  const size_t wsm = sizeof(float) * 4 * (N / n);
+  const size_t wsm = sizeof(float) * 4 * f;
   const int64_t inner2 = (int64_t)N * N, chunk2 = inner2 < 2048 ? inner2 : 2048;
   k_up_axis<<<dim3((unsigned)(3 * n * n), 1), threads, wsm, st>>>(n, N, N, N, t1, t2, nullptr);
   k_up_axis<<<dim3((unsigned)(3 * n), (unsigned)((inner2 + chunk2 - 1) / chunk2)), 256, wsm, st>>>(
