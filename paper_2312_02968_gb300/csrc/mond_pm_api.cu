@@ -650,29 +650,29 @@ int do_bin(mond_pm* h) {
   unsigned nb = (unsigned)((h->N + 255) / 256);
   if (h->N > 0) {
     Timed tm(h, KC_BIN, 32.0 * h->N);
-    parts::k_bin_count<<<nb, 256, 0, h->st>>>(b);
+    CK(launch_early(parts::k_bin_count, nb, 256, 0, h->st, b));
   }
   {
     Timed tm(h, KC_BIN, 4.0 * M);
-    parts::k_scan_reduce<<<nblk, 1024, 0, h->st>>>(h->w.count, M, h->w.bsum);
+    CK(launch_early(parts::k_scan_reduce, nblk, 1024, 0, h->st, h->w.count, M, h->w.bsum));
   }
   {
     Timed tm(h, KC_BIN, 8.0 * nblk);
-    parts::k_scan_blocks<<<1, 1024, 0, h->st>>>(h->w.bsum, nblk);
+    CK(launch_early(parts::k_scan_blocks, 1, 1024, 0, h->st, h->w.bsum, nblk));
   }
   {
     Timed tm(h, KC_BIN, 8.0 * M);
-    parts::k_scan_apply<<<nblk, 1024, 0, h->st>>>(h->w.count, M, h->w.bsum, h->w.cstart);
+    CK(launch_early(parts::k_scan_apply, nblk, 1024, 0, h->st, h->w.count, M, h->w.bsum, h->w.cstart));
   }
   if (h->N > 0) {
     Timed tm(h, KC_BIN, 16.0 * h->N);
-    parts::k_bin_scatter<<<nb, 256, 0, h->st>>>(b);
+    CK(launch_early(parts::k_bin_scatter, nb, 256, 0, h->st, b));
   }
   CK(cudaGetLastError());
   h->count_dirty = false;
   {
     Timed tm(h, KC_BIN, 16.0 * h->ntile);
-    parts::k_tile_work<<<(h->ntile + 255) / 256, 256, 0, h->st>>>(b);
+    CK(launch_early(parts::k_tile_work, (h->ntile + 255) / 256, 256, 0, h->st, b));
   }
   CK(cudaGetLastError());
   return MOND_OK;

@@ -65,6 +65,7 @@ struct BinArgs {
 // Key of each particle, or ncell when it is invalid (cell outside [0, n),
 // offset outside [-1/2, 1/2] or not finite, mass not finite).
 __global__ void k_bin_count(BinArgs a) {
+  kernel_wait();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.N) return;
   int c[3];
@@ -109,6 +110,7 @@ __device__ __forceinline__ int block_excl_scan(int v, int* wsum, int* total) {
 // each block of SCAN_B counters (16-byte loads, a warp reduction, the warps'
 // sums in shared memory).
 __global__ void __launch_bounds__(1024) k_scan_reduce(const int* cnt, int64_t M, int* bsum) {
+  kernel_wait();
   __shared__ int wsum[32];
   const int64_t b0 = (int64_t)blockIdx.x * SCAN_B;
   int s = 0;
@@ -133,6 +135,7 @@ __global__ void __launch_bounds__(1024) k_scan_reduce(const int* cnt, int64_t M,
 }
 
 __global__ void __launch_bounds__(1024) k_scan_blocks(int* bsum, int nblk) {
+  kernel_wait();
   __shared__ int wsum[32];
   const int per = (nblk + 1023) / 1024;
   const int i0 = threadIdx.x * per, i1 = min(nblk, i0 + per);
@@ -149,6 +152,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(int* bsum, int nblk) {
 // cnt and cstart may be the same array (each thread reads its run before
 // writing it); both 16-byte aligned.
 __global__ void __launch_bounds__(1024) k_scan_apply(const int* cnt, int64_t M, const int* bsum, int* cstart) {
+  kernel_wait();
   __shared__ int wsum[32];
   constexpr int PER = SCAN_B / 1024;
   static_assert(PER == 8, "two int4 per thread");
@@ -184,6 +188,7 @@ __global__ void __launch_bounds__(1024) k_scan_apply(const int* cnt, int64_t M, 
 
 // Particles -> sorted positions (the order inside a cell is immaterial).
 __global__ void k_bin_scatter(BinArgs a) {
+  kernel_wait();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.N) return;
   uint32_t k = a.key[i];
@@ -195,6 +200,7 @@ __global__ void k_bin_scatter(BinArgs a) {
 // cells apart in the cell scan, so the reads are spread out). A warp reserves
 // its entries with one atomic per counter.
 __global__ void __launch_bounds__(256) k_tile_work(BinArgs a) {
+  kernel_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
   int ts = 0, te = 0;
   if (t < a.ntile) {

@@ -387,6 +387,8 @@ __global__ void __launch_bounds__(NTX) k_xpass(XArgs a, int64_t nlines) {
   const int tid = threadIdx.x;
   const int64_t line0 = (int64_t)blockIdx.x * C::L;
   for (int i = tid; i < N; i += NTX) tw[i] = a.tw[i];
+  kernel_wait();
+  const auto* const dep = after_wait(a.dep);
   constexpr bool INC = MODE == X_DNU_FIRST || MODE == X_DNU || MODE == X_DMU;  // three components, C2R first
   static_assert(INC || MODE == X_RHO || MODE == X_DRHO, "modes of k_xpass");
   constexpr int nc = INC ? 3 : 1;
@@ -424,7 +426,7 @@ __global__ void __launch_bounds__(NTX) k_xpass(XArgs a, int64_t nlines) {
 #pragma unroll
     for (int k = 0; k < PER; k++) {
       const int i = tid + k * NTX, j = i % C::H, l = i / C::H;
-      if (i < C::L * C::H) u[k] = __ldcs(reinterpret_cast<const ulonglong2*>(a.dep + rbase + (int64_t)l * N + 2 * j));
+      if (i < C::L * C::H) u[k] = __ldcs(reinterpret_cast<const ulonglong2*>(dep + rbase + (int64_t)l * N + 2 * j));
     }
 #pragma unroll
     for (int k = 0; k < PER; k++) {

@@ -27,8 +27,7 @@ cudaError_t launch_x(const XArgs& a, cudaStream_t st) {
   cudaError_t e = set_smem(k_xpass<N, MODE>, sm);
   if (e != cudaSuccess) return e;
   int64_t nlines = (int64_t)N * N;
-  k_xpass<N, MODE><<<(unsigned)(nlines / XCfg<N>::L), NTX, sm, st>>>(a, nlines);
-  return cudaGetLastError();
+  return launch_early(k_xpass<N, MODE>, (unsigned)(nlines / XCfg<N>::L), NTX, sm, st, a, nlines);
 }
 
 template <int MODE>
@@ -38,8 +37,7 @@ cudaError_t launch_xreg(const XArgs& a, cudaStream_t st) {
   cudaError_t e = sm > 48 * 1024 ? set_smem(xreg::k_xreg<N, MODE>, sm) : cudaSuccess;
   if (e != cudaSuccess) return e;
   const dim3 grid(N * N / X::LINES, xreg::ncomp_of(MODE) == 3 ? 1 : a.ncomp);
-  xreg::k_xreg<N, MODE><<<grid, 32 * xreg::WARPS, sm, st>>>(a);
-  return cudaGetLastError();
+  return launch_early(xreg::k_xreg<N, MODE>, grid, 32 * xreg::WARPS, sm, st, a);
 }
 
 template <int MODE>
@@ -132,8 +130,7 @@ cudaError_t launch_yreg(const regpass::YRegArgs& a, int cap, cudaStream_t st) {
   cudaError_t e = sm > 48 * 1024 ? set_smem(regpass::k_yreg<N, KIND>, sm) : cudaSuccess;
   if (e != cudaSuccess) return e;
   const int ntiles = G::TILES * (a.nplain + (PAIR ? 1 : 0));
-  regpass::k_yreg<N, KIND><<<capped(ntiles, ntiles, cap), G::T, sm, st>>>(a, ntiles);
-  return cudaGetLastError();
+  return launch_early(regpass::k_yreg<N, KIND>, capped(ntiles, ntiles, cap), G::T, sm, st, a, ntiles);
 }
 
 template <int MODE, bool FOLD, bool PHI>
@@ -142,8 +139,8 @@ cudaError_t launch_zreg(const regpass::ZRegArgs& a, int cap, cudaStream_t st) {
   const size_t sm = regpass::ZCfg<N, MODE, FOLD, PHI>::smem();
   cudaError_t e = sm > 48 * 1024 ? set_smem(regpass::k_zreg<N, MODE, FOLD, PHI>, sm) : cudaSuccess;
   if (e != cudaSuccess) return e;
-  regpass::k_zreg<N, MODE, FOLD, PHI><<<capped(G::TILES, G::TILES, cap), G::T, sm, st>>>(a, G::TILES);
-  return cudaGetLastError();
+  return launch_early(regpass::k_zreg<N, MODE, FOLD, PHI>, capped(G::TILES, G::TILES, cap), G::T, sm, st, a,
+                      G::TILES);
 }
 }  // namespace
 

@@ -287,6 +287,7 @@ __global__ void __launch_bounds__(YGeo<N, KIND>::T, yctas(N, KIND >= Y_FOLD)) k_
   float2* const sm1 = sm + G::SLOTS;
   table_in(tw, a.tw, 8 * N, threadIdx.x, G::T);
   if (PAIR) table_in(kt, a.kt, 4 * N, threadIdx.x, G::T);
+  kernel_wait();
   bool first = true;
   for (int t0 = blockIdx.x; t0 < ntiles; t0 += gridDim.x) {
     if (!first) __syncthreads();
@@ -483,6 +484,7 @@ __global__ void __launch_bounds__(Geo<N>::T, zctas(N)) k_zreg(ZRegArgs a, int nt
   table_in(tw, a.tw, 8 * N, threadIdx.x, G::T);
   table_in(kv, a.kv, 4 * N, threadIdx.x, G::T);
   table_in(kp, a.kp, 4 * N, threadIdx.x, G::T);
+  kernel_wait();
   const bool mean_in = MODE == Z_FINAL && a.mean == 2, mean_out = MODE == Z_CURL && a.mean == 1;
   const bool use_khat = MODE == Z_SMOOTH || (MODE == Z_FINAL && a.khat);
   bool first = true;

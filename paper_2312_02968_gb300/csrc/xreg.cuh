@@ -239,6 +239,8 @@ __global__ void __launch_bounds__(32 * WARPS, ncomp_of(MODE) == 3 ? 3 : 1) k_xre
   float2* const sl = xsm + N + warp * NC * REGION + l * X::PITCH;
   float2* const spec = a.spec + line * SP + (NC == 1 ? blockIdx.y * a.pstride : 0);
   const int64_t rl = line * N + (NC == 1 ? (int64_t)blockIdx.y * P3 : 0);  // first real sample
+  regpass::table_in(tw, a.tw, 8 * N, threadIdx.x, 32 * WARPS);
+  kernel_wait();
   if constexpr (has_inv(MODE)) {
     const uint64_t pol = tma::policy_evict_first();
 #pragma unroll
@@ -250,7 +252,6 @@ __global__ void __launch_bounds__(32 * WARPS, ncomp_of(MODE) == 3 ? 3 : 1) k_xre
       }
     }
   }
-  regpass::table_in(tw, a.tw, 8 * N, threadIdx.x, 32 * WARPS);
   if (lane < 3) {
     // the real planes the pointwise stage reads, brought into L2 meanwhile (the
     // warp's lines are contiguous)
