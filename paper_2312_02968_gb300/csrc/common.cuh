@@ -29,7 +29,9 @@ enum : uint32_t {
 // an event a launch waits as any other, and a graph's kernels follow each
 // other as closely without it. Solve at 96^3: 290 -> 222 us;
 // force step at 64^3, 1e4 particles: 284 -> 181 us, at 192^3, 4e5 particles:
-// 1.91 -> 1.80 ms. Letting the next kernel start with the first CTAs' end
+// 1.91 -> 1.80 ms; surrogate: inference
+// 64^3 -> 256^3 (34 launches) 581 -> 501 us, training step at 32^3 1.66 -> 1.49
+// ms. Letting the next kernel start with the first CTAs' end
 // instead (launch_dependents at their start) was slower: 250, 260 us, 1.86 ms,
 // and 7% slower with eight systems side by side.
 // ---------------------------------------------------------------------------

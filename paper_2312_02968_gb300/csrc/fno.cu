@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "../../include/mond_fno.h"
+#include "common.cuh"
 #include "internal.h"
 
 namespace {
@@ -97,6 +98,10 @@ template <int CMAX>
 __global__ void __launch_bounds__(256) k_pw(const float* __restrict__ in, int Cin, const uint16_t* __restrict__ W,
                                             const uint16_t* __restrict__ b, int Cout, float* __restrict__ out,
                                             int64_t V, int transpose) {
+  kernel_wait();
+  in = after_wait(in);
+  W = after_wait(W);
+  b = after_wait(b);
   __shared__ __align__(16) float sW[32 * CMAX];
   __shared__ float sb[32];
   for (int e = threadIdx.x; e < Cout * CMAX; e += blockDim.x) {
@@ -156,6 +161,10 @@ __global__ void __launch_bounds__(256, 2) k_pw_mma(const float* __restrict__ in,
                                                    const uint16_t* __restrict__ W, const uint16_t* __restrict__ b,
                                                    int Cout, float* __restrict__ out, int64_t V, int transpose,
                                                    int vec_out) {
+  kernel_wait();
+  in = after_wait(in);
+  W = after_wait(W);
+  b = after_wait(b);
   __shared__ uint16_t sW[32][32 + 8];  // [o][i], zero-padded; row pitch 80 bytes (conflict-free fragments)
   __shared__ float sb[32];
   for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
@@ -190,7 +199,7 @@ __global__ void __launch_bounds__(256, 2) k_pw_mma(const float* __restrict__ in,
 #pragma unroll
         for (int j = 0; j < 2; j++) {
           const int k = 16 * ks + 8 * rr + 2 * q + j;
-          x[ks][rr][j] = k < Cin ? __ldg(reinterpret_cast<const float4*>(in + (int64_t)k * V + v0) + g)
+          x[ks][rr][j] = k < Cin ? *(reinterpret_cast<const float4*>(in + (int64_t)k * V + v0) + g)
                                  : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     float d[MT][4][4];  // [M tile][voxel tile][C fragment: rows g, g + 8, columns 2q, 2q + 1]
@@ -245,6 +254,9 @@ __global__ void __launch_bounds__(256, 2) k_pw_mma(const float* __restrict__ in,
 // 16.5 us at 32^3 (32 x 32 channels); now 9.0 us.
 __global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ dout, int Cout, const float* __restrict__ in,
                                                int Cin, int64_t V, float* dW, float* db, int vec) {
+  kernel_wait();
+  dout = after_wait(dout);
+  in = after_wait(in);
   constexpr int CH = 64, P = CH + 4;
   __shared__ __align__(16) float so[32 * P], si[32 * P];
   const int tid = threadIdx.x, ob = tid >> 4, ib = tid & 15, ntiles = (int)(V / CH);
@@ -257,8 +269,8 @@ __global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ dout, i
       const bool live = row < (k < 2 ? Cout : Cin);
       const float* p = src + (int64_t)row * V + (int64_t)tile * CH + 4 * (tid & 15);
       if (!live) pre[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      else if (vec) pre[k] = __ldg(reinterpret_cast<const float4*>(p));
-      else pre[k] = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+      else if (vec) pre[k] = *(reinterpret_cast<const float4*>(p));
+      else pre[k] = make_float4(*(p), *(p + 1), *(p + 2), *(p + 3));
     }
   };
   float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, bias[2] = {0.f, 0.f};
@@ -380,7 +392,7 @@ __global__ void k_mix_bwd(const float2* __restrict__ gt, const float2* __restric
 // through shared memory, as eight modes are the 64 bytes that a channel keeps
 // together. A lane per channel with 4-byte loads and 8-byte strided spectra:
 // 17.8 us forward, 74 us backward at M = 16 (67 and 335 MB); now 13.2 us
-// and 58 us (5.8 TB/s).
+// and 56 us (6.0 TB/s).
 constexpr int MK = 8;   // modes per CTA
 constexpr int MP = 34;  // pitch of a mode's channels: eight modes and two channels in distinct banks
 __device__ __forceinline__ float2 wr_wi(uint32_t w) {
@@ -388,7 +400,7 @@ __device__ __forceinline__ float2 wr_wi(uint32_t w) {
 }
 __device__ __forceinline__ void load_modes(float2 (*s)[MP], const float2* __restrict__ in, int k0, int K) {
   const int m = threadIdx.x % MK, j = threadIdx.x / MK;
-  s[m][j] = k0 + m < K ? __ldg(in + (int64_t)j * K + k0 + m) : make_float2(0.f, 0.f);
+  s[m][j] = k0 + m < K ? *(in + (int64_t)j * K + k0 + m) : make_float2(0.f, 0.f);
 }
 __device__ __forceinline__ void store_modes(const float2 (*s)[MP], float2* __restrict__ out, int k0, int K) {
   const int m = threadIdx.x % MK, j = threadIdx.x / MK;
@@ -396,6 +408,9 @@ __device__ __forceinline__ void store_modes(const float2 (*s)[MP], float2* __res
 }
 __global__ void __launch_bounds__(256) k_mix_fwd32(const float2* __restrict__ s, const uint4* __restrict__ R,
                                                    float2* __restrict__ t, int K) {
+  kernel_wait();
+  s = after_wait(s);
+  R = after_wait(R);
   __shared__ float2 sS[MK][MP], sO[MK][MP];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k0 = blockIdx.x * MK, k = k0 + warp;
   uint4 w[8];
@@ -434,10 +449,18 @@ __global__ void __launch_bounds__(256) k_mix_fwd32(const float2* __restrict__ s,
 __global__ void __launch_bounds__(256) k_mix_bwd32(const float2* __restrict__ gt, const float2* __restrict__ s,
                                                    const uint4* __restrict__ R, float2* __restrict__ gs,
                                                    float4* __restrict__ dR, int K, int M, float invV) {
+  kernel_wait();
+  gt = after_wait(gt);
+  s = after_wait(s);
+  R = after_wait(R);
+  dR = after_wait(dR);
   __shared__ float2 sG[MK][MP], sS[MK][MP], sO[MK][MP];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k0 = blockIdx.x * MK, k = k0 + warp;
   const bool live = k < K;
   const int64_t base = (int64_t)k * 256 + lane;
+  uint4 w[8];  // before any store: they are not moved past one
+#pragma unroll
+  for (int jj = 0; jj < 8; jj++) w[jj] = live ? __ldcs(R + base + 32 * jj) : make_uint4(0, 0, 0, 0);
   load_modes(sG, gt, k0, K);
   load_modes(sS, s, k0, K);
   __syncthreads();
@@ -451,12 +474,10 @@ __global__ void __launch_bounds__(256) k_mix_bwd32(const float2* __restrict__ gt
   }
 #pragma unroll
   for (int half = 0; half < 2; half++) {
-    uint4 w[4];
     float4 d[4][2];
 #pragma unroll
     for (int q = 0; q < 4; q++) {
       const int64_t r = base + 32 * (4 * half + q);
-      w[q] = live ? __ldg(R + r) : make_uint4(0, 0, 0, 0);
       d[q][0] = live ? __ldcs(dR + 2 * r) : make_float4(0.f, 0.f, 0.f, 0.f);
       d[q][1] = live ? __ldcs(dR + 2 * r + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -464,7 +485,7 @@ __global__ void __launch_bounds__(256) k_mix_bwd32(const float2* __restrict__ gt
     for (int q = 0; q < 4; q++) {
       const int jj = 4 * half + q;
       const float2 x = sS[warp][4 * jj + (lane >> 3)];
-      const uint32_t u[4] = {w[q].x, w[q].y, w[q].z, w[q].w};
+      const uint32_t u[4] = {w[jj].x, w[jj].y, w[jj].z, w[jj].w};
       p[jj] = make_float2(0.f, 0.f);
 #pragma unroll
       for (int c = 0; c < 4; c++) {
@@ -506,8 +527,11 @@ bool mix32(int C, const void* R, const void* dR) {
 
 __global__ void __launch_bounds__(256) k_gelu_bwd(const float4* __restrict__ z, const float4* __restrict__ dv,
                                                   float4* __restrict__ dz, int64_t n4) {
+  kernel_wait();
+  z = after_wait(z);
+  dv = after_wait(dv);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-    const float4 a = __ldg(z + i), b = __ldg(dv + i);
+    const float4 a = *(z + i), b = *(dv + i);
     float4 d;
     gelu_t(a.x, &d.x);
     gelu_t(a.y, &d.y);
@@ -527,6 +551,10 @@ __global__ void k_sumsq(const float* t, int64_t n, double* out) {
 
 __global__ void k_loss(const float* y, const float* t, float* dy, int64_t n, const double* tnorm, float weight,
                        double* loss) {
+  kernel_wait();
+  y = after_wait(y);
+  t = after_wait(t);
+  tnorm = after_wait(tnorm);
   __shared__ double s_inv;
   if (threadIdx.x == 0) s_inv = 1.0 / fmax(*tnorm, 1e-300);
   __syncthreads();
@@ -550,6 +578,9 @@ __global__ void k_loss(const float* y, const float* t, float* dy, int64_t n, con
 // sums) -> 96 us, 5.6 TB/s; 786432 floats: 40 -> 6 us.
 __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, int64_t n4, const float* __restrict__ tail,
                                                   int ntail, double* out) {
+  kernel_wait();
+  t = after_wait(t);
+  tail = after_wait(tail);
   __shared__ double part[8];
   float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f}, top = 0.f;
   auto add = [&](int k, float x) {
@@ -562,7 +593,7 @@ __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, 
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
 #pragma unroll 4
   for (int64_t i = i0; i < n4; i += stride) {
-    const float4 x = __ldg(t + i);
+    const float4 x = *(t + i);
     add(0, x.x);
     add(1, x.y);
     add(2, x.z);
@@ -582,7 +613,7 @@ __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, 
     r = (double)s[0] + (double)c[0];
   } else {
     for (int64_t i = i0; i < n4; i += stride) {
-      const float4 x = __ldg(t + i);
+      const float4 x = *(t + i);
       r += (double)x.x * x.x + (double)x.y * x.y + (double)x.z * x.z + (double)x.w * x.w;
     }
     if (i0 < ntail) r += (double)tail[i0] * tail[i0];
@@ -622,6 +653,12 @@ __device__ __forceinline__ void adam1(const AdamArgs& a, float scale, float& p, 
 // (two kernels) -> 0.68 ms, 6.7 TB/s.
 __global__ void __launch_bounds__(256) k_adam(int64_t n, float* p, float* g, float* m, float* v, uint16_t* pb,
                                               AdamArgs a, int vec) {
+  kernel_wait();
+  p = after_wait(p);
+  g = after_wait(g);
+  m = after_wait(m);
+  v = after_wait(v);
+  a.sumsq = after_wait(a.sumsq);
   __shared__ float s_scale;  // one thread takes the FP64 square root
   if (threadIdx.x == 0) s_scale = adam_scale(a);
   __syncthreads();
@@ -720,6 +757,10 @@ __global__ void k_coarsen(int N, int n, const float* __restrict__ fine, const fl
 __global__ void __launch_bounds__(256, 6) k_coarsen4(int N, int n, const float4* __restrict__ fine,
                                                   const float4* __restrict__ fine2, float* __restrict__ coarse,
                                                   const float* __restrict__ scale) {
+  kernel_wait();
+  fine = after_wait(fine);
+  fine2 = after_wait(fine2);
+  scale = after_wait(scale);
   extern __shared__ __align__(16) float sx[];  // [RY][N]
   const int f = N / n, TX = N / 4, RY = blockDim.y, xq = threadIdx.x, ry = threadIdx.y;
   const int row = (blockIdx.z * n + blockIdx.y) * n + blockIdx.x;
@@ -768,8 +809,8 @@ void launch_coarsen(int N, int n, int ncomp, const float* fine, const float* fin
                     const float* scale, cudaStream_t st) {
   if (N % 4 == 0 && N <= 1024 && ncomp < 65536 && aligned16(fine) && aligned16(fine2)) {
     const int f = N / n, TX = N / 4, RY = std::min(f * f, 256 / TX);
-    k_coarsen4<<<dim3(n, n, ncomp), dim3(TX, RY), sizeof(float) * N * RY, st>>>(
-        N, n, reinterpret_cast<const float4*>(fine), reinterpret_cast<const float4*>(fine2), coarse, scale);
+    launch_early(k_coarsen4, dim3(n, n, ncomp), dim3(TX, RY), sizeof(float) * N * RY, st, N, n,
+                 reinterpret_cast<const float4*>(fine), reinterpret_cast<const float4*>(fine2), coarse, scale);
     return;
   }
   const int threads = N < 256 ? ((N + 31) / 32) * 32 : 256;
@@ -777,6 +818,9 @@ void launch_coarsen(int N, int n, int ncomp, const float* fine, const float* fin
 }
 
 __global__ void k_input(int n, float a0, const float* g, const double* sumsq, float* x, float* scale_out) {
+  kernel_wait();
+  g = after_wait(g);
+  sumsq = after_wait(sumsq);
   const int64_t V = (int64_t)n * n * n;
   __shared__ float s_rms;  // one thread a CTA does the FP64 arithmetic
   if (threadIdx.x == 0) s_rms = (float)sqrt(fmax(*sumsq / (3.0 * V), 1e-60));
@@ -898,6 +942,9 @@ __global__ void __launch_bounds__(256) k_up3(int n, int N, const float4* __restr
                        s * (w.x * a.z + w.y * b.z + w.z * d.z + w.w * e.z),
                        s * (w.x * a.w + w.y * b.w + w.z * d.w + w.w * e.w));
   };
+  kernel_wait();
+  in = after_wait(in);
+  scale = after_wait(scale);
   // x: weights and coarse cells of this thread's four positions X0 + k of the
   // coarse cell i, which lie past the coarse position i - 1 or, from f/2 on, i
   const float s = *scale;
@@ -916,7 +963,7 @@ __global__ void __launch_bounds__(256) k_up3(int n, int N, const float4* __restr
     const int jz = jz0 + step, k0 = step ? 3 : 0;
     for (int r = 4 * k0 + ry * f + q; r < 16; r += RY * f) {
       const int z = wrap(jz - 1 + r / 4, n), y = wrap(jy - 1 + r % 4, n);
-      sC[(4 * ((step + r / 4) & 3) + r % 4) * n4 + i4] = __ldg(in + (((int64_t)c * n + z) * n + y) * n4 + i4);
+      sC[(4 * ((step + r / 4) & 3) + r % 4) * n4 + i4] = *(in + (((int64_t)c * n + z) * n + y) * n4 + i4);
     }
     __syncthreads();
     for (int k = k0 + ry; k < 4; k += RY) {
@@ -983,8 +1030,8 @@ unsigned grid_stride(int64_t n) {
 void sumsq(const float* t, int64_t n, double* out, cudaStream_t st) {
   if (aligned16(t))
     // eight vectors a thread at least: a thread ends with FP64 sums
-    k_gradnorm<<<grid_stride((n + 31) / 32), TB, 0, st>>>(reinterpret_cast<const float4*>(t), n / 4, t + n / 4 * 4,
-                                                        (int)(n % 4), out);
+    launch_early(k_gradnorm, grid_stride((n + 31) / 32), TB, 0, st, reinterpret_cast<const float4*>(t), n / 4,
+                 t + n / 4 * 4, (int)(n % 4), out);
   else
     k_sumsq<<<grid_stride(n), TB, 0, st>>>(t, n, out);
 }
@@ -1032,8 +1079,8 @@ void dft3(const Shape& s, const Work& w, const float* v, float2* out, cudaStream
   by_size(n, M, [&](auto nx, auto mx, auto full) {
     constexpr int NX = nx.value, MX = mx.value;
     constexpr bool FULL = full.value;
-    dft::k_xy_fwd<NX, MX, FULL><<<plane_grid(np), dft::TH, dft::smem_xy_fwd(n, M), st>>>(v, w.b, n, M, np);
-    dft::k_z_fwd<NX, MX, FULL><<<gz, dft::TH, sz, st>>>(w.b, out, n, M, Iz);
+    launch_early(dft::k_xy_fwd<NX, MX, FULL>, plane_grid(np), dft::TH, dft::smem_xy_fwd(n, M), st, v, w.b, n, M, np);
+    launch_early(dft::k_z_fwd<NX, MX, FULL>, gz, dft::TH, sz, st, w.b, out, n, M, Iz);
   });
 }
 
@@ -1048,8 +1095,9 @@ void idft3(const Shape& s, const Work& w, const float2* in, float* z, float* v, 
   by_size(n, M, [&](auto nx, auto mx, auto full) {
     constexpr int NX = nx.value, MX = mx.value;
     constexpr bool FULL = full.value;
-    dft::k_z_inv<NX, MX, FULL><<<gz, dft::TH, sz, st>>>(in, w.b, n, M, Iz);
-    dft::k_xy_inv<NX, MX, FULL><<<plane_grid(np), dft::TH, dft::smem_xy_inv(n, M), st>>>(w.b, z, v, n, M, w0, w1, act, np);
+    launch_early(dft::k_z_inv<NX, MX, FULL>, gz, dft::TH, sz, st, in, w.b, n, M, Iz);
+    launch_early(dft::k_xy_inv<NX, MX, FULL>, plane_grid(np), dft::TH, dft::smem_xy_inv(n, M), st, w.b, z, v, n, M,
+                 w0, w1, act, np);
   });
 }
 
@@ -1057,13 +1105,13 @@ void pw(const float* in, int Cin, const uint16_t* W, const uint16_t* b, int Cout
         int transpose, cudaStream_t st) {
   const unsigned g = grid_stride(V);
   if (Cin <= 4) {
-    k_pw<4><<<g, TB, 0, st>>>(in, Cin, W, b, Cout, out, V, transpose);
+    launch_early(k_pw<4>, g, TB, 0, st, in, Cin, W, b, Cout, out, V, transpose);
   } else {
     // tensor cores: one warp per 32 voxels a step (V = n^3 is a multiple of 64), two CTAs per SM
     const unsigned gm = (unsigned)std::min<int64_t>((V / 32 + 7) / 8, 152 * 2);
     const int vec = aligned16(out);
-    if (Cout <= 16) k_pw_mma<1><<<gm, TB, 0, st>>>(in, Cin, W, b, Cout, out, V, transpose, vec);
-    else k_pw_mma<2><<<gm, TB, 0, st>>>(in, Cin, W, b, Cout, out, V, transpose, vec);
+    if (Cout <= 16) launch_early(k_pw_mma<1>, gm, TB, 0, st, in, Cin, W, b, Cout, out, V, transpose, vec);
+    else launch_early(k_pw_mma<2>, gm, TB, 0, st, in, Cin, W, b, Cout, out, V, transpose, vec);
   }
 }
 
@@ -1118,7 +1166,7 @@ int mond_fno_forward(mond_fno_shape sh, const uint16_t* P, const float* x, float
     dft3(s, w, vl, shat, st);
     const uint16_t* R = P + s.off_R(l);
     if (mix32(C, R, nullptr))
-      k_mix_fwd32<<<(s.K + MK - 1) / MK, TB, 0, st>>>(shat, reinterpret_cast<const uint4*>(R), w.c, s.K);
+      launch_early(k_mix_fwd32, (s.K + MK - 1) / MK, TB, 0, st, shat, reinterpret_cast<const uint4*>(R), w.c, s.K);
     else
       k_mix_fwd<<<warps_grid, TB, 0, st>>>(shat, R, w.c, C, s.K);
     idft3(s, w, w.c, zl, w.v + (l + 1) * CV, false, l + 1 < s.L ? 1 : 2, st);
@@ -1140,8 +1188,8 @@ int mond_fno_backward(mond_fno_shape sh, const uint16_t* P, const float* x, cons
   const unsigned gw = (unsigned)std::min<int64_t>(V / 64, 152);
   const unsigned warps_grid = (unsigned)(((int64_t)s.K * 32 + TB - 1) / TB);
   // projection
-  k_wgrad<<<gw, TB, 0, st>>>(dy, 3, w.v + s.L * CV, C, V, grad + s.off_Q(), grad + s.off_q(),
-                              aligned16(dy) && aligned16(w.v + s.L * CV));
+  launch_early(k_wgrad, gw, TB, 0, st, dy, 3, w.v + s.L * CV, C, V, grad + s.off_Q(), grad + s.off_q(),
+               aligned16(dy) && aligned16(w.v + s.L * CV));
   float* dv = w.dv;
   float* dv2 = w.dv2;
   pw(dy, 3, P + s.off_Q(), nullptr, C, dv, V, 1, st);
@@ -1150,14 +1198,13 @@ int mond_fno_backward(mond_fno_shape sh, const uint16_t* P, const float* x, cons
     const float* zl = w.z + l * CV;
     const float* dz = dv;  // the last layer has no activation
     if (l + 1 < s.L) {
-      k_gelu_bwd<<<grid_stride(CV / 4), TB, 0, st>>>(reinterpret_cast<const float4*>(zl),
-                                                      reinterpret_cast<const float4*>(dv),
-                                                      reinterpret_cast<float4*>(w.dz), CV / 4);
+      launch_early(k_gelu_bwd, grid_stride(CV / 4), TB, 0, st, reinterpret_cast<const float4*>(zl),
+                   reinterpret_cast<const float4*>(dv), reinterpret_cast<float4*>(w.dz), CV / 4);
       dz = w.dz;
     }
     // pointwise part
-    k_wgrad<<<gw, TB, 0, st>>>(dz, C, vl, C, V, grad + s.off_W(l), grad + s.off_b(l),
-                              aligned16(dz) && aligned16(vl));
+    launch_early(k_wgrad, gw, TB, 0, st, dz, C, vl, C, V, grad + s.off_W(l), grad + s.off_b(l),
+                 aligned16(dz) && aligned16(vl));
     pw(dz, C, P + s.off_W(l), nullptr, C, dv2, V, 1, st);
     // spectral part: G_t = (a/V) DFT(dz), through the mixing adjoint, back with the adjoint transform
     dft3(s, w, dz, w.c, st);
@@ -1165,8 +1212,8 @@ int mond_fno_backward(mond_fno_shape sh, const uint16_t* P, const float* x, cons
     const uint16_t* R = P + s.off_R(l);
     float* dR = grad + s.off_R(l);
     if (mix32(C, R, dR))
-      k_mix_bwd32<<<(s.K + MK - 1) / MK, TB, 0, st>>>(w.c, shat, reinterpret_cast<const uint4*>(R), w.d,
-                                                      reinterpret_cast<float4*>(dR), s.K, M, 1.f / (float)V);
+      launch_early(k_mix_bwd32, (s.K + MK - 1) / MK, TB, 0, st, w.c, shat, reinterpret_cast<const uint4*>(R), w.d,
+                   reinterpret_cast<float4*>(dR), s.K, M, 1.f / (float)V);
     else
       k_mix_bwd<<<warps_grid, TB, 0, st>>>(w.c, shat, R, w.d, dR, C, s.K, M, 1.f / (float)V);
     idft3(s, w, w.d, dv2, nullptr, true, 0, st);
@@ -1175,8 +1222,8 @@ int mond_fno_backward(mond_fno_shape sh, const uint16_t* P, const float* x, cons
     dv2 = t;
   }
   // lift
-  k_wgrad<<<gw, TB, 0, st>>>(dv, C, x, 4, V, grad + s.off_P(), grad + s.off_p(),
-                              aligned16(dv) && aligned16(x));
+  launch_early(k_wgrad, gw, TB, 0, st, dv, C, x, 4, V, grad + s.off_P(), grad + s.off_p(),
+               aligned16(dv) && aligned16(x));
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -1187,7 +1234,7 @@ int mond_fno_loss(int64_t count, const float* y, const float* t, float* dy, floa
   double* tn = loss_acc + 1;  // scratch slot after the accumulator
   cudaMemsetAsync(tn, 0, sizeof(double), st);
   sumsq(t, count, tn, st);
-  k_loss<<<grid_stride(count), TB, 0, st>>>(y, t, dy, count, tn, weight, loss_acc);
+  launch_early(k_loss, grid_stride(count), TB, 0, st, y, t, dy, count, tn, weight, loss_acc);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -1201,7 +1248,7 @@ int mond_fno_adam_cast(int64_t count, float* p, float* g, float* m, float* v, fl
   sumsq(g, count, scratch, st);
   const int vec = aligned16(p) && aligned16(g) && aligned16(m) && aligned16(v) &&
                   (reinterpret_cast<uintptr_t>(pb) & 7) == 0;
-  k_adam<<<vec ? grid : grid_stride(count), TB, 0, st>>>(count, p, g, m, v, pb, a, vec);
+  launch_early(k_adam, vec ? grid : grid_stride(count), TB, 0, st, count, p, g, m, v, pb, a, vec);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -1226,7 +1273,7 @@ int mond_fno_input(int N, int n, float a0, const float* gN, float* x, float* sca
   double* acc = reinterpret_cast<double*>(scale_out + 2);  // scale_out must have room for 2 + 2 floats
   cudaMemsetAsync(acc, 0, sizeof(double), st);
   sumsq(x, 3 * V, acc, st);
-  k_input<<<grid_stride(V), TB, 0, st>>>(n, a0, x, acc, x, scale_out);
+  launch_early(k_input, grid_stride(V), TB, 0, st, n, a0, x, acc, x, scale_out);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -1241,8 +1288,8 @@ int mond_fno_output(int N, int n, const float* y, const float* scale, float* H, 
   if (f > 64) return -1;
   cudaStream_t st = (cudaStream_t)stream;
   if (f % 4 == 0 && n % 4 == 0 && N <= 512 && aligned16(y) && aligned16(H)) {
-    k_up3<<<dim3(n, n / UPZ, 3 * (f / 4)), dim3(N / 4, 256 / (N / 4)), smem_up3(n, N), st>>>(
-        n, N, reinterpret_cast<const float4*>(y), reinterpret_cast<float4*>(H), scale);
+    launch_early(k_up3, dim3(n, n / UPZ, 3 * (f / 4)), dim3(N / 4, 256 / (N / 4)), smem_up3(n, N), st, n, N,
+                 reinterpret_cast<const float4*>(y), reinterpret_cast<float4*>(H), scale);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
   }
   float* t1 = (float*)scratch;              // [3 n n][N]   x upsampled

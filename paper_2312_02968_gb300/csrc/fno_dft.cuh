@@ -85,11 +85,13 @@ __global__ void __launch_bounds__(TH, 2) k_xy_fwd(const float* __restrict__ v, f
     for (int k = 0; k < FIT; k++) {
       const int y = fy + k * (TH / HX);
       if (fx < H && y < n) {
-        pre[k][0] = __ldg(src + y * n + fx);
-        pre[k][1] = __ldg(src + y * n + fx2);
+        pre[k][0] = src[y * n + fx];
+        pre[k][1] = src[y * n + fx2];
       }
     }
   };
+  kernel_wait();
+  v = after_wait(v);
   if ((int)blockIdx.x < nplanes) fetch(blockIdx.x);
   for (int plane = blockIdx.x; plane < nplanes; plane += gridDim.x) {
 #pragma unroll
@@ -216,11 +218,14 @@ __global__ void __launch_bounds__(TH, 2) k_xy_inv(const float2* __restrict__ in,
     for (int k = 0; k < FIT; k++) {
       const int f = ff + k * (TH / MX);
       if (fk < M && f < M) {
-        pre[k][0] = __ldg(src + f * M + fk);
-        pre[k][1] = __ldg(src + (f ? 2 * M - f : M) * M + fk);
+        pre[k][0] = src[f * M + fk];
+        pre[k][1] = src[(f ? 2 * M - f : M) * M + fk];
       }
     }
   };
+  kernel_wait();
+  in = after_wait(in);
+  z = after_wait(z);
   if ((int)blockIdx.x < nplanes) fetch(blockIdx.x);
   for (int plane = blockIdx.x; plane < nplanes; plane += gridDim.x) {
 #pragma unroll
@@ -339,17 +344,19 @@ __global__ void __launch_bounds__(TH) k_z_fwd(const float2* __restrict__ in, flo
   float2* cs = reinterpret_cast<float2*>(sT + H * (M + 1));
   in += (int64_t)blockIdx.y * n * I;
   out += (int64_t)blockIdx.y * 2 * M * I;
+  circle(cs, n);
+  kernel_wait();
+  in = after_wait(in);
   float2 p[4], q[4];
 #pragma unroll
   for (int k = 0; k < 4; k++) {
     const int z = warp + 8 * k;
     p[k] = q[k] = make_float2(0.f, 0.f);
     if (z < H && i < I) {
-      p[k] = __ldg(in + (int64_t)z * I + i);
-      q[k] = __ldg(in + (int64_t)(z ? n - z : H) * I + i);
+      p[k] = in[(int64_t)z * I + i];
+      q[k] = in[(int64_t)(z ? n - z : H) * I + i];
     }
   }
-  circle(cs, n);
   __syncthreads();
   pair_table(sT, cs, H, n, M);
 #pragma unroll
@@ -399,17 +406,19 @@ __global__ void __launch_bounds__(TH) k_z_inv(const float2* __restrict__ in, flo
   float2* cs = reinterpret_cast<float2*>(sT + (H + 1) * (M + 1));
   in += (int64_t)blockIdx.y * 2 * M * I;
   out += (int64_t)blockIdx.y * n * I;
+  circle(cs, n);
+  kernel_wait();
+  in = after_wait(in);
   float2 p[4], q[4];
 #pragma unroll
   for (int k = 0; k < 4; k++) {
     const int f = warp + 8 * k;
     p[k] = q[k] = make_float2(0.f, 0.f);
     if (f < M && i < I) {
-      p[k] = __ldg(in + (int64_t)f * I + i);
-      q[k] = __ldg(in + (int64_t)(f ? 2 * M - f : M) * I + i);
+      p[k] = in[(int64_t)f * I + i];
+      q[k] = in[(int64_t)(f ? 2 * M - f : M) * I + i];
     }
   }
-  circle(cs, n);
   __syncthreads();
   pair_table(sT, cs, H + 1, n, M);
 #pragma unroll
