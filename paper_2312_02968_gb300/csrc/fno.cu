@@ -315,8 +315,8 @@ __global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ dout, i
 __device__ __forceinline__ float gelu_t(float z, float* dgdz) {
   const float k0 = 0.7978845608028654f, k1 = 0.044715f;
   const float u = k0 * (z + k1 * z * z * z);
-  const float t = expf(fminf(-2.f * u, 80.f)), s = 1.f / (1.f + t);
-  if (dgdz) *dgdz = s + z * (t * s * s) * (2.f * k0) * (1.f + 3.f * k1 * z * z);
+  const float t = expf(-2.f * u), s = 1.f / (1.f + t);  // t = inf: s = 0
+  if (dgdz) *dgdz = s + z * (fminf(t, 3e38f) * s * s) * (2.f * k0) * (1.f + 3.f * k1 * z * z);
   return z * s;
 }
 
