@@ -24,16 +24,15 @@ enum : uint32_t {
 // nothing that an earlier kernel writes is read and nothing is written. What
 // others write is read after the wait by plain loads, or through a pointer from
 // after_wait: the compiler may move read-only loads and __ldcs, whose assembly
-// it does not take for a memory access, past the wait. Every thread waits, so a completed
-// kernel implies that all before it have completed. After a copy, a memset or
-// an event a launch waits as any other, and a graph's kernels follow each
-// other as closely without it. Solve at 96^3: 290 -> 222 us;
-// force step at 64^3, 1e4 particles: 284 -> 181 us, at 192^3, 4e5 particles:
-// 1.91 -> 1.80 ms; surrogate: inference
-// 64^3 -> 256^3 (34 launches) 581 -> 501 us, training step at 32^3 1.66 -> 1.49
-// ms. Letting the next kernel start with the first CTAs' end
-// instead (launch_dependents at their start) was slower: 250, 260 us, 1.86 ms,
-// and 7% slower with eight systems side by side.
+// it does not take for a memory access, past the wait. Every thread waits, so a
+// completed kernel implies that all before it have completed. After a copy, a
+// memset or an event a launch waits as any other.
+// Solve at 96^3: 290 -> 222 us; force step at 64^3, 1e4 particles: 284 -> 181
+// us, at 192^3, 4e5 particles: 1.91 -> 1.80 ms; surrogate: inference 64^3 ->
+// 256^3 (34 launches) 581 -> 501 us, training step at 32^3 1.66 -> 1.49 ms. A
+// graph's kernels follow each other as closely without it (no change). Letting
+// the next kernel in when the first has started (launch_dependents) was slower:
+// 250 us, 260 us, 1.86 ms, and 7% with eight systems side by side.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void kernel_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename T>

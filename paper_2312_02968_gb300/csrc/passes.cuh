@@ -3,8 +3,8 @@
 //
 // Data layout in HBM:
 //  real planes     float [z][y][x], N^3 values (x fastest)
-//  spectral planes float2 [z][y][kx], kx = 0..N/2 in rows of SP = N/2 + 2
-//                  complex (16-byte aligned rows); y and z are either real
+//  spectral planes float2 [z][y][kx], kx = 0..N/2 in rows of SP = N/2 + 4
+//                  complex (32-byte aligned rows); y and z are either real
 //                  coordinates or frequencies depending on the stage.
 // A 3-D transform is an x-pass (R2C / C2R on contiguous lines), a y-pass and
 // a z-pass (C2C on strided lines, tiles of P adjacent kx columns). The
