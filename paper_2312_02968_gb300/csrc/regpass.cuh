@@ -142,10 +142,21 @@ struct Geo {
 };
 
 // CTAs per SM the passes are compiled for (registers: 65536 / (T ctas); 1: no
-// limit). At 256, z 3 / 4: divergence-free 0.116 / 0.126 ms (spills), folded
-// final 0.104 / 0.121 ms; pair y-passes 4 / 5: 0.073 / 0.071 and 0.068 / 0.070.
-constexpr int zctas(int n) { return n == 256 ? 3 : 1; }
-constexpr int yctas(int n, bool pair) { return n == 256 && pair ? 4 : 1; }
+// limit). Without a limit the compiler takes 184 to 199 registers for the
+// z-passes of 128 and 192, two CTAs per SM, and 144 to 150 for the pair
+// y-passes, three. Per side, of a K = 4 solve:
+//   192, z 3: divergence-free 57 -> 50 us, final 51 -> 43 (4: no gain);
+//        pair y 4: fold 39 -> 34 us, unfold 34 -> 31 (5: no gain); plain y 7:
+//        a force step 1701 -> 1695 us;
+//   128, a step of two particles: z 3: 543 -> 534 us, and pair y 4: 529,
+//        and z 4: 515 (5: 524);
+//   256, z 3 / 4: divergence-free 116 / 126 us (spills), folded final 104 /
+//        121; pair y 4 / 5: 73 / 71 and 68 / 70;
+//   64, 96: no difference.
+constexpr int zctas(int n) { return n == 128 ? 4 : n == 192 || n == 256 ? 3 : 1; }
+constexpr int yctas(int n, bool pair) {
+  return pair ? (n >= 128 && n <= 256 ? 4 : 1) : n == 192 ? 7 : 1;
+}
 
 // The exchange slot of butterfly j, value r, of this thread's sequence.
 template <class G>

@@ -72,6 +72,11 @@ constexpr size_t smem_bytes() {
   return sizeof(float2) * (N + (size_t)WARPS * ncomp_of(MODE) * Geo<N>::REGION);
 }
 
+// CTAs per SM the three-component modes are compiled for. 192: 4 (128 instead of
+// 136 registers) nu 95 -> 81 us; 128: 5, eight systems side by side 1% less (6:
+// 1% more); 256: what shared memory admits; 64, 96: more made no difference.
+constexpr int xctas(int n) { return n == 192 ? 4 : n == 128 ? 5 : 3; }
+
 // 16-byte asynchronous copy whose source lines leave L2 first (read once).
 __device__ __forceinline__ void copy16_stream(void* dst, const void* src, uint64_t policy) {
   asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(tma::smem_addr(dst)), "l"(src),
@@ -226,7 +231,7 @@ __device__ __forceinline__ void factors(const XArgs& a, float2* m2) {
 }
 
 template <int N, int MODE>
-__global__ void __launch_bounds__(32 * WARPS, ncomp_of(MODE) == 3 ? 3 : 1) k_xreg(XArgs a) {
+__global__ void __launch_bounds__(32 * WARPS, ncomp_of(MODE) == 3 ? xctas(N) : 1) k_xreg(XArgs a) {
   using X = Geo<N>;
   constexpr int A0 = X::A0, A1 = X::A1, TL = X::TL, H = X::H, SP = X::SP, REGION = X::REGION;
   constexpr int NC = ncomp_of(MODE);
