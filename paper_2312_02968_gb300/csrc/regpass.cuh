@@ -152,10 +152,16 @@ struct Geo {
 //        and z 4: 515 (5: 524);
 //   256, z 3 / 4: divergence-free 116 / 126 us (spills), folded final 104 /
 //        121; pair y 4 / 5: 73 / 71 and 68 / 70;
+//   384 (T = 192: one CTA per SM without a limit, both kinds), a K = 4 solve:
+//        13.1 ms; z 2: 12.0, and pair y 2: 10.9, 3: 10.6, and plain y 4: 10.2
+//        (16 threads a sequence with limits to match: 10.5);
+//   512, pair y 3 instead of 2: a K = 4 solve 23.7 -> 23.4 ms (z 3, pair y 4,
+//        plain y 5: no gain);
 //   64, 96: no difference.
-constexpr int zctas(int n) { return n == 128 ? 4 : n == 192 || n == 256 ? 3 : 1; }
+constexpr int zctas(int n) { return n == 128 ? 4 : n == 192 || n == 256 ? 3 : n == 384 ? 2 : 1; }
 constexpr int yctas(int n, bool pair) {
-  return pair ? (n >= 128 && n <= 256 ? 4 : 1) : n == 192 ? 7 : 1;
+  if (pair) return n >= 384 ? 3 : n >= 128 ? 4 : 1;
+  return n == 192 ? 7 : n == 384 ? 4 : 1;
 }
 
 // The exchange slot of butterfly j, value r, of this thread's sequence.
