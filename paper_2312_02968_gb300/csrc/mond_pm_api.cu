@@ -310,15 +310,16 @@ struct mond_pm {
     int n_iter, warm, keep_phi, track_dh, pipelined, chunk, gather_mode, ext_axis;
     double ext_mass;
     int64_t N;
-    const void* cell;
+    const void *cell, *off, *vel, *mass;
+    int kacc;
     const void* inc;
     int cycle_mean, fold, grid_cap, vel_wait;
     bool operator==(const GraphKey& o) const {
       return dt == o.dt && n_iter == o.n_iter && warm == o.warm && keep_phi == o.keep_phi &&
              track_dh == o.track_dh && pipelined == o.pipelined && chunk == o.chunk &&
              gather_mode == o.gather_mode && ext_axis == o.ext_axis && ext_mass == o.ext_mass && N == o.N &&
-             cell == o.cell && inc == o.inc && cycle_mean == o.cycle_mean && fold == o.fold &&
-             grid_cap == o.grid_cap && vel_wait == o.vel_wait;
+             cell == o.cell && off == o.off && vel == o.vel && mass == o.mass && kacc == o.kacc && inc == o.inc &&
+             cycle_mean == o.cycle_mean && fold == o.fold && grid_cap == o.grid_cap && vel_wait == o.vel_wait;
     }
   } gkey{};
   int64_t glaunches = 0;
@@ -1505,6 +1506,14 @@ int step_checks(mond_pm_t h, int n_iter, int warm) {
   return MOND_OK;
 }
 
+// Everything a captured step's launches were made from: a graph is replayed
+// only while this is what it was at the capture.
+mond_pm::GraphKey graph_key(const mond_pm* h, double dt, int n_iter, int warm) {
+  return {dt,          n_iter,      warm,          h->keep_phi,   h->track_dh,         h->pipelined, h->chunk,
+          h->gather_mode, h->ext_axis, h->ext_mass, h->N,          h->cell,             h->off,       h->vel,
+          h->mass,     h->kacc,     h->inc.dep0,   h->cycle_mean, use_fold(h) ? 1 : 0, h->grid_cap,  h->vel_wait};
+}
+
 // Enqueue the step on h->st while h->st is being captured into a graph.
 int capture_into(mond_pm_t h, double dt, int n_iter, int warm) { return step_direct(h, dt, n_iter, warm); }
 
@@ -1512,9 +1521,7 @@ int step_graph(mond_pm_t h, double dt, int n_iter, int warm) {
   if (!capturable(h->st)) return fail(h, MOND_ESTATE, "a captured step needs a non-default stream");
   int rc = step_checks(h, n_iter, warm);
   if (rc) return rc;
-  const mond_pm::GraphKey key{dt,       n_iter,          warm,        h->keep_phi, h->track_dh, h->pipelined,
-                              h->chunk, h->gather_mode, h->ext_axis, h->ext_mass, h->N,         h->cell,
-                              h->inc.dep0, h->cycle_mean, use_fold(h) ? 1 : 0, h->grid_cap, h->vel_wait};
+  const mond_pm::GraphKey key = graph_key(h, dt, n_iter, warm);
   if (!h->gexec || !(key == h->gkey)) {
     if (h->gexec) {
       cudaGraphExecDestroy(h->gexec);
@@ -1631,9 +1638,7 @@ int mond_pm_batch_step(mond_pm_batch_t b, double dt, int n_steps, int n_iter, in
     if (rc) return rc;
   }
   std::vector<mond_pm::GraphKey> keys;
-  for (auto h : b->hs)
-    keys.push_back({dt, n_iter, warm, h->keep_phi, h->track_dh, h->pipelined, h->chunk, h->gather_mode, h->ext_axis,
-                    h->ext_mass, h->N, h->cell, h->inc.dep0});
+  for (auto h : b->hs) keys.push_back(graph_key(h, dt, n_iter, warm));
   bool same = b->gexec && keys.size() == b->keys.size();
   for (size_t i = 0; same && i < keys.size(); i++) same = keys[i] == b->keys[i];
   if (!same) {
