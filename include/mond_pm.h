@@ -193,7 +193,8 @@ int mond_pm_deposit(mond_pm_t h);
 
 /* Use a mesh density instead of a deposit for the next solves: rho (device
  * float32, n_f^3, mass per s^3) is copied in; the next mond_pm_deposit
- * replaces it. Particle calls (gather, push) need a deposit. */
+ * replaces it. Particle calls (gather, push) need a deposit of the bound
+ * particles where they are (MOND_ESTATE otherwise). */
 int mond_pm_set_density(mond_pm_t h, const float* rho);
 
 /* Field solve (Sect. 2.1 iteration; App. Flow steps 3-9) on the last

@@ -273,6 +273,7 @@ struct mond_pm {
   const float* mass = nullptr;
   int kacc = 0;
   bool have_dep = false, have_solve = false, have_khat = false, have_smooth = false, density_given = false;
+  bool binned = false;    // the work list and the order are those of the bound particles where they are now
   bool gn_valid = false;  // w.gN holds the Newton field of the current density
   bool have_fields = false;  // w.gN and w.acc hold the fields of a solve
   int gather_mode = 0;        // MOND_OPT_GATHER: 0 Eq. gi, 1 / 3 interpolation order
@@ -728,6 +729,7 @@ int do_deposit(mond_pm* h) {
   CK(cudaGetLastError());
   h->have_dep = true;
   h->have_solve = false;
+  h->binned = true;
   h->density_given = false;
   h->gn_valid = false;
   return MOND_OK;
@@ -763,6 +765,11 @@ int do_gather(mond_pm* h, float* g_out, double dt, int kick, int drift) {
     return fail(h, MOND_ESTATE, h->gather_mode ? "the interpolating gather needs a solve with n_iter >= 1 made with "
                                                  "MOND_OPT_GATHER set"
                                                : "the acceleration mesh is smoothed: solve again with MOND_OPT_GATHER 0");
+  if (!h->binned) {
+    // a solve of a density set directly does not bin the particles: the lists would be stale or unset memory
+    if (h->N > 0) return fail(h, MOND_ESTATE, "the particles have not been deposited since they were bound or moved");
+    return MOND_OK;
+  }
   if (h->gather_mode) {
     Timed tm(h, KC_GATHER, 3.0 * real_bytes(h) + 64.0 * h->N);
     const int nbk = h->sms * 8;
@@ -1346,6 +1353,7 @@ int mond_pm_bind_particles(mond_pm_t h, int64_t N, int32_t* cell, float* offset,
   h->kacc = 62 - (emax - 126) - L;
   h->have_dep = false;
   h->have_solve = false;
+  h->binned = false;
   return MOND_OK;
 }
 
@@ -1459,6 +1467,7 @@ int mond_pm_gather_push(mond_pm_t h, double dt) {
   if (rc == MOND_OK) {
     h->have_dep = false;  // particles moved: the binning is stale
     h->have_solve = false;
+    h->binned = false;
   }
   return rc;
 }
