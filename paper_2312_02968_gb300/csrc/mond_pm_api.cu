@@ -254,7 +254,22 @@ struct TimedLaunch {
   cudaEvent_t a, b;
 };
 
-struct mond_pm {
+// What the calls have left in the workspace. A step being captured runs none of
+// its launches, and a replayed one none of its host code, so both set this apart
+// from the calls that do (step_graph, mond_pm_batch_step).
+struct StepState {
+  bool have_dep = false, have_solve = false, density_given = false;
+  bool binned = false;        // the work list and the order are those of the bound particles where they are now
+  bool count_dirty = true;    // the binning's cell counters may be nonzero
+  bool gn_valid = false;      // w.gN holds the Newton field of the current density
+  bool have_fields = false;   // w.gN and w.acc hold the fields of a solve
+  bool acc_smoothed = false;  // w.acc holds the node-smoothed field (final pass with the smoothing spectrum)
+  bool inc_valid = false;     // the base (dep0, gN, Hs, gM0, acc) is that of the last solve
+  int inc_kacc = 0, inc_gather = 0, inc_keep_phi = 0;
+  int last_iters = 0;
+};
+
+struct mond_pm : StepState {
   int n, npad, nf;
   double box, s, a0, G, sigma;
   int mu_kind, r, nb, nrows = 0;
@@ -272,14 +287,10 @@ struct mond_pm {
   float* vel = nullptr;
   const float* mass = nullptr;
   int kacc = 0;
-  bool have_dep = false, have_solve = false, have_khat = false, have_smooth = false, density_given = false;
-  bool binned = false;    // the work list and the order are those of the bound particles where they are now
-  bool gn_valid = false;  // w.gN holds the Newton field of the current density
-  bool have_fields = false;  // w.gN and w.acc hold the fields of a solve
+  bool have_khat = false, have_smooth = false;
   int gather_mode = 0;        // MOND_OPT_GATHER: 0 Eq. gi, 1 / 3 interpolation order
   int ext_axis = -1;          // external-field dipole layer (mond_pm_set_dipole_layer), -1 none
   double ext_mass = 0.0;
-  bool acc_smoothed = false;  // w.acc holds the node-smoothed field (final pass with the smoothing spectrum)
   // incremental solve (mond_pm_set_increment_workspace): the base deposit, the
   // base g_M and the increment's Newton field, in a caller-owned buffer
   struct IncWs {
@@ -287,12 +298,9 @@ struct mond_pm {
     float* gM0 = nullptr;
     float* dgN = nullptr;
   } inc;
-  bool inc_valid = false;  // the base (dep0, gN, Hs, gM0, acc) is that of the last solve
-  int inc_kacc = 0, inc_gather = 0, inc_keep_phi = 0;
   int keep_phi = 0, track_dh = 0, use_graph = 0, timing = 0, pipelined = 1;
   int lost_tile = -1;  // MOND_OPT_TEST_LOST_LOAD: tile of the next pipelined y-pass whose copy is not issued
   int cycle_mean = 0;  // MOND_OPT_CYCLE_MEAN
-  bool count_dirty = true;  // the binning's cell counters may be nonzero
   int fold = 1;        // MOND_OPT_FOLD (used where the pipelined passes run and the size allows it)
   int grid_cap = 0;    // MOND_OPT_GRID_CAP: CTAs of a persistent kernel at most (0: all that fit)
   // mond_pm_step_host: the velocities go in on a copy stream of their own while
@@ -323,6 +331,7 @@ struct mond_pm {
              cycle_mean == o.cycle_mean && fold == o.fold && grid_cap == o.grid_cap && vel_wait == o.vel_wait;
     }
   } gkey{};
+  StepState gafter;  // what a replay leaves
   int64_t glaunches = 0;
   // TMA views of the spectral buffers for the staged y-pass of the bounded-wait tests
   tma::TensorMap map_wy, map_ay;
@@ -331,7 +340,6 @@ struct mond_pm {
   std::vector<cudaEvent_t> evpool;  // recycled events
   int64_t st_launch[KC_COUNT] = {};
   double st_ms[KC_COUNT] = {}, st_bytes[KC_COUNT] = {};
-  int last_iters = 0;
   int64_t launches = 0;
   std::string err;
 };
@@ -1531,12 +1539,14 @@ int step_graph(mond_pm_t h, double dt, int n_iter, int warm) {
   int rc = step_checks(h, n_iter, warm);
   if (rc) return rc;
   const mond_pm::GraphKey key = graph_key(h, dt, n_iter, warm);
-  if (!h->gexec || !(key == h->gkey)) {
+  // (a graph captured with clean cell counters does not clear them)
+  if (!h->gexec || !(key == h->gkey) || h->count_dirty) {
     if (h->gexec) {
       cudaGraphExecDestroy(h->gexec);
       h->gexec = nullptr;
     }
     const int64_t l0 = h->launches;
+    const StepState before = *h;
     CK(cudaStreamBeginCapture(h->st, cudaStreamCaptureModeRelaxed));
     h->capturing = true;
     rc = capture_into(h, dt, n_iter, warm);
@@ -1545,6 +1555,8 @@ int step_graph(mond_pm_t h, double dt, int n_iter, int warm) {
     const cudaError_t e = cudaStreamEndCapture(h->st, &g);  // always ends the capture
     h->glaunches = h->launches - l0;
     h->launches = l0;
+    h->gafter = *h;
+    static_cast<StepState&>(*h) = before;  // nothing has run yet
     if (rc || e != cudaSuccess) {
       if (g) cudaGraphDestroy(g);
       return rc ? rc : fail(h, MOND_ECUDA, "step capture: %s", cudaGetErrorString(e));
@@ -1558,6 +1570,7 @@ int step_graph(mond_pm_t h, double dt, int n_iter, int warm) {
     h->gkey = key;
   }
   CK(cudaGraphLaunch(h->gexec, h->st));
+  static_cast<StepState&>(*h) = h->gafter;
   h->launches += h->glaunches;
   return MOND_OK;
 }
@@ -1586,6 +1599,7 @@ struct mond_pm_batch {
   double dt = 0;
   int n_iter = -1, warm = -1;
   std::vector<mond_pm::GraphKey> keys;
+  std::vector<StepState> after;  // what a replay leaves of each member
   int64_t glaunches = 0, launches = 0;
 };
 
@@ -1649,7 +1663,7 @@ int mond_pm_batch_step(mond_pm_batch_t b, double dt, int n_steps, int n_iter, in
   std::vector<mond_pm::GraphKey> keys;
   for (auto h : b->hs) keys.push_back(graph_key(h, dt, n_iter, warm));
   bool same = b->gexec && keys.size() == b->keys.size();
-  for (size_t i = 0; same && i < keys.size(); i++) same = keys[i] == b->keys[i];
+  for (size_t i = 0; same && i < keys.size(); i++) same = keys[i] == b->keys[i] && !b->hs[i]->count_dirty;
   if (!same) {
     if (b->gexec) {
       cudaGraphExecDestroy(b->gexec);
@@ -1658,7 +1672,11 @@ int mond_pm_batch_step(mond_pm_batch_t b, double dt, int n_steps, int n_iter, in
     // one graph: fork from the batch stream to every handle's stream, one step
     // of each system on its own stream, join back
     std::vector<int64_t> l0(n);
-    for (int i = 0; i < n; i++) l0[i] = b->hs[i]->launches;
+    std::vector<StepState> before;
+    for (int i = 0; i < n; i++) {
+      l0[i] = b->hs[i]->launches;
+      before.push_back(*b->hs[i]);
+    }
     cudaError_t e = cudaStreamBeginCapture(b->st, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) return fail(b->hs[0], MOND_ECUDA, "batch capture: %s", cudaGetErrorString(e));
     int rc = MOND_OK;
@@ -1681,9 +1699,12 @@ int mond_pm_batch_step(mond_pm_batch_t b, double dt, int n_steps, int n_iter, in
     cudaGraph_t g = nullptr;
     const cudaError_t ee = cudaStreamEndCapture(b->st, &g);
     b->glaunches = 0;
+    b->after.clear();
     for (int i = 0; i < n; i++) {
       b->glaunches += b->hs[i]->launches - l0[i];
       b->hs[i]->launches = l0[i];
+      b->after.push_back(*b->hs[i]);
+      static_cast<StepState&>(*b->hs[i]) = before[i];  // nothing has run yet
     }
     if (rc || e != cudaSuccess || ee != cudaSuccess) {
       if (g) cudaGraphDestroy(g);
@@ -1701,6 +1722,7 @@ int mond_pm_batch_step(mond_pm_batch_t b, double dt, int n_steps, int n_iter, in
   for (int k = 0; k < n_steps; k++) {
     const cudaError_t e = cudaGraphLaunch(b->gexec, b->st);
     if (e != cudaSuccess) return fail(b->hs[0], MOND_ECUDA, "batch graph launch: %s", cudaGetErrorString(e));
+    for (int i = 0; i < n; i++) static_cast<StepState&>(*b->hs[i]) = b->after[i];
   }
   b->launches += b->glaunches * n_steps;
   return MOND_OK;

@@ -73,3 +73,51 @@ def test_no_particles_and_a_density(B):
     h.gather_push(0.1)  # (a push ends the solve's validity)
     h.sync()
     h.close()
+
+
+@pytest.mark.parametrize("how", ["graph", "batch"])
+def test_a_replay_ends_a_solve_as_a_step_does(B, how):
+    h, t = system(B)
+    if how == "graph":
+        h.set_option(B.OPT_USE_GRAPH, 1)
+        step = lambda: h.step(0.5, 2)
+    else:
+        b = B.Batch([h])
+        step = lambda: (b.step(0.5, n_steps=1, n_iter=2), b.sync())
+    step()  # captured and run
+    h.deposit()
+    h.solve_field(1)
+    assert torch.isfinite(h.gather()).all()
+    step()  # replayed: the particles have moved
+    refused(B, h.gather)
+    refused(B, lambda: h.solve_field(1))
+    assert h.diagnostics()["n_iter_done"] == 2
+    if how == "batch":
+        b.step(0.5, n_steps=0, n_iter=3)  # captured, not run
+        assert h.diagnostics()["n_iter_done"] == 2
+        b.close()
+    h.close()
+
+
+def test_a_capture_that_fails_leaves_nothing_behind(B):
+    # the workspace of a handle that has never binned holds whatever was there
+    junk = torch.full((B.workspace_bytes(N_SIDE, 1, 1.0, 3000) + 256,), 0x5A, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    del junk
+    h, t = system(B)
+    h.set_option(B.OPT_USE_GRAPH, 1)
+    h.set_option(B.OPT_CYCLE_MEAN, 1)
+    h.set_option(B.OPT_PIPELINED, 0)
+    refused(B, lambda: h.step(0.5, 2))  # the mean needs the other passes: after the deposit was captured
+    refused(B, lambda: h.solve_field(2))  # no deposit has run
+    h.set_option(B.OPT_PIPELINED, 1)
+    h.step(0.5, 2)
+    h.sync()
+    h2, t2 = system(B)
+    h2.set_option(B.OPT_CYCLE_MEAN, 1)
+    h2.step(0.5, 2)
+    h2.sync()
+    for a, b in zip(t, t2):
+        assert torch.equal(a, b)
+    h.close()
+    h2.close()
