@@ -21,6 +21,7 @@ constexpr int CHUNK = 1024;   // default particles per work item (runtime: the a
 // 0.16, 0.18 / 0.14, 0.17 / 0.13, 0.17 / 0.13, 0.16 / 0.14, 0.20 / 0.16 ms for
 // 4e5 of a Plummer sphere on 192^3 (sigma 1).
 constexpr int SPARSE = 16;
+constexpr int SMS = 152;      // SMs of the GPU
 constexpr int QHALF = 32768;  // offset quantisation: q = round(offset * 2^16) + 32768
 constexpr int SCAN_B = 8192;  // elements per block of the key scan
 
@@ -572,13 +573,18 @@ __device__ __forceinline__ void deposit_range(const DepArgs& a, int q0, int q1, 
 // Runs f(first entry, past the last, first step of taps, steps between) over
 // the list of the particles of sparse tiles: two entries at a time (one while
 // the grid has a warp for each) taken by the grid's warps from a counter, or,
-// with a CTA for each entry, the warps of a CTA sharing its taps (a system of
-// a few particles: the latency of a warp's walk over the ball is all its time).
+// up to `wide` entries (a CTA for each on the whole GPU), the warps of a CTA
+// sharing its taps (a system of a few particles: the latency of a warp's walk
+// over the ball is all its time). The two sum a particle's taps in different
+// orders, so the choice is one of the list alone, not of the CTAs launched.
 template <typename F>
-__device__ __forceinline__ void for_sparse(const int* nsparse, int* counter, F&& f) {
+__device__ __forceinline__ void for_sparse(const int* nsparse, int* counter, int wide, F&& f) {
   const int n = __ldg(nsparse), nw = blockDim.x >> 5;
-  if (n <= (int)gridDim.x) {
-    if ((int)blockIdx.x < n) f(blockIdx.x, blockIdx.x + 1, threadIdx.x >> 5, nw);
+  if (n <= wide) {
+    for (int r = blockIdx.x; r < n; r += gridDim.x) {
+      if (r != (int)blockIdx.x) __syncthreads();  // the CTA's sums of the entry before have been read
+      f(r, r + 1, threadIdx.x >> 5, nw);
+    }
     return;
   }
   const int run = n <= (int)gridDim.x * nw ? 1 : 2;
@@ -702,7 +708,8 @@ __global__ void __launch_bounds__(DEP_NT, dep_ctas(R)) k_deposit(DepArgs a) {
       atomicAdd((unsigned long long*)(a.dep + (gz * a.n + gy) * a.n + gx), v);
     }
   }
-  for_sparse(a.work.count + 2, a.work_counter + 1, [&](int r0, int r1, int first, int step) { deposit_sparse<R>(a, r0, r1, first, step); });
+  for_sparse(a.work.count + 2, a.work_counter + 1, SMS * dep_ctas(R),
+             [&](int r0, int r1, int first, int step) { deposit_sparse<R>(a, r0, r1, first, step); });
 }
 template <int R>
 constexpr size_t dep_smem_bytes() {
@@ -1029,7 +1036,7 @@ __global__ void __launch_bounds__(gat_threads(R), gat_ctas(R)) k_gather_push(Gat
     gather_range<R>(a, q0, q1, ox, oy, oz, sa, sz, lr, stage + warp);
   }
   __shared__ float part[gat_threads(R) / 32][4];
-  for_sparse(a.work.count + 2, a.work_counter + 1, [&](int r0, int r1, int first, int step) {
+  for_sparse(a.work.count + 2, a.work_counter + 1, SMS * gat_ctas(R), [&](int r0, int r1, int first, int step) {
     gather_sparse<R>(a, r0, r1, first, step, part);
   });
 }
