@@ -97,8 +97,8 @@ enum {
   MOND_OPT_TIMING = 4,    /* value 1: bracket every launch with CUDA events (see mond_pm_kernel_stats) */
   MOND_OPT_PIPELINED = 5, /* value 1 (default): y/z passes with their transforms in registers;
                              0: in shared memory, with plain loads (same results up to FP32 rounding order) */
-  MOND_OPT_CHUNK = 6,     /* particles per deposit/gather work item at most: a power of two in 256..4096
-                             (default 1024; a small system's items are smaller; same results) */
+  MOND_OPT_CHUNK = 6,     /* particles per deposit/gather work item: a power of two in 256..4096; 1024 (the
+                             default) stands for 1024 or fewer, as the number of particles asks (same results) */
   MOND_OPT_GATHER = 7,    /* force at the particles. 0 (default): Eq. gi, the ball sum at each particle.
                              1 or 3: the mesh-interpolating gather -- the final pass of a solve (n_iter >= 1)
                              also multiplies the acceleration spectrum by the smoothing spectrum, so that
@@ -351,10 +351,10 @@ int64_t mond_pm_batch_kernel_launches(mond_pm_batch_t b);
 int mond_pm_batch_destroy(mond_pm_batch_t b);
 
 /* Autotuner: time `trials` steps of length zero (which leave the particles
- * exactly as they are; the H state is reset) for each work-item size in
- * {512, 1024, 2048, 4096} and each pass variant (MOND_OPT_PIPELINED 0/1) on
- * the handle's stream, keep the fastest and report it (either out pointer may
- * be NULL). Synchronises. */
+ * exactly as they are; the H state is reset) for each MOND_OPT_CHUNK in
+ * {512, 1024, 2048, 4096} (but one that the default 1024 already stands for)
+ * and each pass variant (MOND_OPT_PIPELINED 0/1) on the handle's stream, keep
+ * the fastest and report it (either out pointer may be NULL). Synchronises. */
 int mond_pm_autotune(mond_pm_t h, int n_iter, int trials, int64_t* chosen_chunk, int* chosen_pipelined);
 
 /* One time step through host memory: copies cell/offset/vel of the N bound

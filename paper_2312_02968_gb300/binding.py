@@ -390,11 +390,13 @@ class MondPM:
 
 def tune_key(h: MondPM, n_iter: int) -> str:
     """Key of a tuning result: the GPU, the FFT-domain side, the particle count
-    (rounded to a power of two), the kernel width and the iteration count."""
+    (rounded to a power of two), the kernel width, the iteration count and the
+    rule that the stored sizes were measured under (2: sizes other than the
+    default are exact)."""
     torch = h.torch
     n = h.particles[3].numel() if getattr(h, "particles", None) else 0
     return (f"{torch.cuda.get_device_name(h.device)}|nf={h.nf}|N~2^{max(n, 1).bit_length()}|"
-            f"sigma={h.kernel_width:g}|K={int(n_iter)}")
+            f"sigma={h.kernel_width:g}|K={int(n_iter)}|rule=2")
 
 
 def autotune(h: MondPM, n_iter: int = 4, trials: int = 3, cache: str | None = None):

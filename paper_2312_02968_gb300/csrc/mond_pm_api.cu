@@ -619,11 +619,13 @@ int persistent_ctas(const mond_pm* h, int per_sm) {
   return (h->grid_cap > 0 && h->grid_cap < g) ? h->grid_cap : g;
 }
 
-// Particles per work item: the option's value, halved while the particles
-// would make fewer than four full items per SM (down to 64: an item's fixed
-// cost, staging and flushing its tile, is that of about 30 particles).
+// Particles per work item: the option's value, or by default 1024, halved while
+// the particles would make fewer than four full items per SM (down to 64: an
+// item's fixed cost, staging and flushing its tile, is that of about 30
+// particles).
 int chunk_of(const mond_pm* h) {
   int c = h->chunk;
+  if (c != parts::CHUNK) return c;
   while (c > MIN_CHUNK && h->N < (int64_t)c * 4 * h->sms) c >>= 1;
   return c;
 }
@@ -1743,7 +1745,9 @@ int mond_pm_batch_sync(mond_pm_batch_t b) {
 
 // Per-handle choice of the work-item size and the pass variant: each candidate
 // is timed over a few steps of length zero (deposit, solve, gather and a push
-// that moves nothing), so the particle state is left exactly as it was.
+// that moves nothing), so the particle state is left exactly as it was. The
+// default comes first and a size that is the same as its own is left out, so
+// that no two candidates differ by noise alone.
 int mond_pm_autotune(mond_pm_t h, int n_iter, int trials, int64_t* chosen_chunk, int* chosen_pipelined) {
   if (!h || trials < 1) return MOND_EINVAL;
   int rc = step_checks(h, n_iter, MOND_WARM_NONE);
@@ -1755,9 +1759,12 @@ int mond_pm_autotune(mond_pm_t h, int n_iter, int trials, int64_t* chosen_chunk,
   h->timing = 0;
   float best = 1e30f;
   int best_chunk = h->chunk, best_pipe = h->pipelined;
-  const int chunks[] = {512, 1024, 2048, 4096};
+  const int chunks[] = {parts::CHUNK, 512, 2048, 4096};
+  h->chunk = parts::CHUNK;
+  const int automatic = chunk_of(h);
   for (int pipe = 0; pipe < 2 && !rc; pipe++)
     for (int c : chunks) {
+      if (c == automatic && c != parts::CHUNK) continue;
       h->pipelined = pipe;
       h->chunk = c;
       rc = step_direct(h, 0.0, n_iter, MOND_WARM_NONE);  // warm-up
