@@ -249,9 +249,11 @@ __global__ void __launch_bounds__(256, 2) k_pw_mma(const float* __restrict__ in,
 // dW[o][i] += sum_v dout[o][v] in[i][v]; db[o] += sum_v dout[o][v].
 // Tiles of 64 voxels in shared memory, the next one's loads in flight; a
 // thread owns the rows ob, ob + 16 and the columns ib, ib + 16 of dW, four
-// voxels a read. A CTA per SM: each adds its 1056 sums to the same words, and
-// with four CTAs per SM those atomics and one product per two reads took
-// 16.5 us at 32^3 (32 x 32 channels); now 9.0 us.
+// voxels a read. A tile is summed by itself and then added to the running sums,
+// so that a chain of additions is 64 long and not 64 times the CTA's tiles. A
+// CTA per SM: each adds its 1056 sums to the same words, and with four CTAs per
+// SM those atomics and one product per two reads took 16.5 us at 32^3 (32 x 32
+// channels); now 9.0 us.
 __global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ dout, int Cout, const float* __restrict__ in,
                                                int Cin, int64_t V, float* dW, float* db, int vec) {
   kernel_wait();
@@ -282,6 +284,7 @@ __global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ dout, i
       *reinterpret_cast<float4*>((k < 2 ? so : si) + ((tid >> 4) + 16 * (k & 1)) * P + 4 * (tid & 15)) = pre[k];
     __syncthreads();
     if (tile + (int)gridDim.x < ntiles) fetch(tile + gridDim.x);
+    float s[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, sb[2] = {0.f, 0.f};
 #pragma unroll 4
     for (int c = 0; c < CH; c += 4) {
       float4 a[2], x[2];
@@ -289,13 +292,19 @@ __global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ dout, i
       for (int r = 0; r < 2; r++) {
         a[r] = *reinterpret_cast<const float4*>(so + (ob + 16 * r) * P + c);
         x[r] = *reinterpret_cast<const float4*>(si + (ib + 16 * r) * P + c);
-        bias[r] += (a[r].x + a[r].y) + (a[r].z + a[r].w);
+        sb[r] += (a[r].x + a[r].y) + (a[r].z + a[r].w);
       }
 #pragma unroll
       for (int r = 0; r < 2; r++)
 #pragma unroll
         for (int t = 0; t < 2; t++)
-          acc[r][t] = fmaf(a[r].x, x[t].x, fmaf(a[r].y, x[t].y, fmaf(a[r].z, x[t].z, fmaf(a[r].w, x[t].w, acc[r][t]))));
+          s[r][t] = fmaf(a[r].x, x[t].x, fmaf(a[r].y, x[t].y, fmaf(a[r].z, x[t].z, fmaf(a[r].w, x[t].w, s[r][t]))));
+    }
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+      bias[r] += sb[r];
+#pragma unroll
+      for (int t = 0; t < 2; t++) acc[r][t] += s[r][t];
     }
   }
 #pragma unroll
