@@ -578,13 +578,17 @@ __global__ void k_loss(const float* y, const float* t, float* dy, int64_t n, con
   if ((threadIdx.x & 31) == 0) atomicAdd(loss, s * inv * weight);
 }
 
-// Sum of the squares of many floats (16-byte aligned), added to out. Bound by
-// the read: every product is exact as two floats and the sums are compensated
-// (FP32 pairs, about 48 bits), as this GPU's FP64 rate is a 64th of its FP32
-// rate. A thread whose values leave the range where that is exact enough
-// (past 1e18 in size, all below 1e-12, infinities, NaNs) sums them in FP64.
-// 134e6 floats: 252 us (FP64
-// sums) -> 96 us, 5.6 TB/s; 786432 floats: 40 -> 6 us.
+// Sum of the squares of floats (16-byte aligned), added to out. Bound by the
+// read: every product is exact as two floats and the sums are compensated (FP32
+// pairs, about 48 bits), as this GPU's FP64 rate is a 64th of its FP32 rate. A
+// thread whose values leave the range where that is exact enough (past 1e18 in
+// size, all below 1e-12, infinities, NaNs) sums them in FP64. Over many
+// threads the pairs' roundings average out: against the exact sum 1e-15 (rms)
+// for 98304 floats and 1.2e-15 for 5e6, where FP64 sums and an unordered add
+// per warp are off by 1.5e-15 and 6.5e-15. Below PAIRS vectors they do not
+// (1.5e-15 against 2e-16 for 64 floats) and all is FP64, one vector a thread.
+// 134e6 floats: 252 us (FP64 sums) -> 96 us, 5.6 TB/s; 786432 floats: 40 -> 6 us.
+constexpr int64_t PAIRS = 16384;
 __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, int64_t n4, const float* __restrict__ tail,
                                                   int ntail, double* out) {
   kernel_wait();
@@ -600,18 +604,21 @@ __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, 
     top = fmaxf(top, fabsf(x));
   };
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool pairs = n4 >= PAIRS;
+  if (pairs) {
 #pragma unroll 4
-  for (int64_t i = i0; i < n4; i += stride) {
-    const float4 x = *(t + i);
-    add(0, x.x);
-    add(1, x.y);
-    add(2, x.z);
-    add(3, x.w);
+    for (int64_t i = i0; i < n4; i += stride) {
+      const float4 x = *(t + i);
+      add(0, x.x);
+      add(1, x.y);
+      add(2, x.z);
+      add(3, x.w);
+    }
+    if (i0 < ntail) add(0, tail[i0]);
   }
-  if (i0 < ntail) add(0, tail[i0]);
   double r = 0.0;
   const float sum = (s[0] + s[1]) + (s[2] + s[3]);
-  if (isfinite(sum) && top < 1e18f && (top == 0.f || top > 1e-12f)) {
+  if (pairs && isfinite(sum) && top < 1e18f && (top == 0.f || top > 1e-12f)) {
     // the four sums as one float pair, then one FP64 addition a thread
 #pragma unroll
     for (int k = 1; k < 4; k++) {
@@ -1038,8 +1045,8 @@ unsigned grid_stride(int64_t n) {
 // *out += the sum of the squares of t.
 void sumsq(const float* t, int64_t n, double* out, cudaStream_t st) {
   if (aligned16(t))
-    // eight vectors a thread at least: a thread ends with FP64 sums
-    launch_early(k_gradnorm, grid_stride((n + 31) / 32), TB, 0, st, reinterpret_cast<const float4*>(t), n / 4,
+    // pairs: eight vectors a thread at least, as a thread ends with FP64 sums
+    launch_early(k_gradnorm, grid_stride(n / 4 >= PAIRS ? (n + 31) / 32 : (n + 3) / 4), TB, 0, st, reinterpret_cast<const float4*>(t), n / 4,
                  t + n / 4 * 4, (int)(n % 4), out);
   else
     k_sumsq<<<grid_stride(n), TB, 0, st>>>(t, n, out);
