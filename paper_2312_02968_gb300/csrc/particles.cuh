@@ -798,7 +798,10 @@ struct GatPasses {
 // pair of particles). Taps outside the ball are held as 0. A lane's sums of a
 // particle go to shared memory and are added over the lanes for GBATCH
 // particles at a time, 32 values by one lane, instead of a shuffle reduction
-// per particle; the lane that adds them kicks and drifts that axis. 0.93 ->
+// per particle; the lane that adds them kicks and drifts that axis. Added one
+// after the other they raised the rms error of a force by 4 to 6%; pairwise, in
+// 0.3% more time, it is that of the reduction (1.18, 1.25, 1.12 and 1.22e-7 at
+// sigma 0.75, 1, 1.5 and 2). 0.93 ->
 // 0.66 ms for 1e6 particles of an isothermal sphere on 256^3 (sigma 1.5), 3.56
 // -> 1.99 ms for 1e7 of a mixture of spheres (sigma 1), 77 -> 18 us for 10007
 // on 64^3.
@@ -910,13 +913,21 @@ __device__ __forceinline__ void gather_range(const GatArgs& a, int q0, int q1, i
     }
     __syncwarp();
     if (lp < cnt) {
-      float g = 0.f;
+      // added pairwise, lanes 16 apart first: five roundings deep, as a
+      // reduction over the warp
+      const float4* q = reinterpret_cast<const float4*>(st->sum[lane]);
+      float4 g[4];
 #pragma unroll
-      for (int j = 0; j < 8; j++) {
-        const float4 q = reinterpret_cast<const float4*>(st->sum[lane])[j];
-        g += (q.x + q.y) + (q.z + q.w);
+      for (int j = 0; j < 4; j++) {
+        const float4 u = q[j], w = q[j + 4];
+        g[j] = make_float4(u.x + w.x, u.y + w.y, u.z + w.z, u.w + w.w);
       }
-      gather_push1(a, i, lax, g, c, o, v);
+#pragma unroll
+      for (int k = 2; k > 0; k >>= 1)
+#pragma unroll
+        for (int j = 0; j < k; j++)
+          g[j] = make_float4(g[j].x + g[j + k].x, g[j].y + g[j + k].y, g[j].z + g[j + k].z, g[j].w + g[j + k].w);
+      gather_push1(a, i, lax, (g[0].x + g[0].z) + (g[0].y + g[0].w), c, o, v);
     }
   }
 }
