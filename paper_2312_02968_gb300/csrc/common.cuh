@@ -106,14 +106,3 @@ __device__ __forceinline__ int wrapi(int i, int n) {
 }
 
 __device__ __forceinline__ void set_status(uint32_t* st, uint32_t bit) { atomicOr(st, bit); }
-
-// ---------------------------------------------------------------------------
-// Mesh geometry passed by value to every pass.
-// ---------------------------------------------------------------------------
-struct MeshGeom {
-  int n;          // FFT-domain side n_f
-  int sp;         // spectral row stride in complex elements (n/2 + 2)
-  int64_t plane;  // spectral plane stride in complex elements (n * n * sp)
-  int64_t cells;  // n^3
-  float s;        // pixel width
-};

@@ -110,21 +110,6 @@ __device__ __forceinline__ void store_3d(const TensorMap* map, int x, int y, int
                : "memory");
 }
 
-// 4-D tiled load and store (used with the component as its own dimension).
-__device__ __forceinline__ void load_4d(void* dst, const TensorMap* map, int x, int c, int y, int z, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-      "%5}], [%6];" ::"r"(smem_addr(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(c), "r"(y), "r"(z), "r"(smem_addr(bar))
-      : "memory");
-}
-__device__ __forceinline__ void store_4d(const TensorMap* map, int x, int c, int y, int z, const void* src) {
-  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(x), "r"(c), "r"(y), "r"(z), "r"(smem_addr(src))
-               : "memory");
-}
-
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 
 // Wait until at most N committed store groups still read shared memory.
