@@ -83,7 +83,7 @@ enum {
   MOND_EOVERFLOW = -4, /* fixed-point bound violated (cannot happen for N < 2^31) */
   MOND_EDOMAIN = -5,   /* a particle's cell or offset is outside the domain; it was skipped */
   MOND_ENAN = -6,      /* a non-finite value appeared in a field or a particle */
-  MOND_ETIMEOUT = -7,  /* a bounded device wait gave up (kernel returned early) */
+  MOND_ETIMEOUT = -7,  /* a bounded device wait gave up (MOND_OPT_TEST_LOST_LOAD: no other call waits on the device) */
   MOND_ESTATE = -8     /* call out of order (no particles bound, no solve yet, ...) */
 };
 
@@ -107,12 +107,14 @@ enum {
                              that field at its position: an approximation of Eq. gi whose error the caller
                              measures against variant 0. A gather whose variant disagrees with the mesh
                              the last solve made fails with MOND_ESTATE. */
-  MOND_OPT_TEST_LOST_LOAD = 8, /* tests of the bounded device waits only. value t + 1 (t >= 0): in the next
-                             pipelined y-pass the tile copy of tile t is never issued, so the wait for it
-                             gives up after a short bound, the CTA waits for the copy it did issue and
-                             stops, and the next synchronising call returns MOND_ETIMEOUT (the fields of
-                             that solve are invalid; the handle stays usable). One-shot: cleared by that
-                             launch. 0: off. Needs MOND_OPT_PIPELINED 1 and no graph replay. */
+  MOND_OPT_TEST_LOST_LOAD = 8, /* tests of the bounded device waits only. The passes of a solve wait for nothing
+                             on the device; this option puts a kernel that does in the place of the next
+                             plain y-pass (tiles staged by TMA copies). value t + 1 (t >= 0): the copy of
+                             tile t is never issued, so the wait for it gives up after a short bound, the CTA
+                             waits for the copy it did issue and stops, and the next synchronising call
+                             returns MOND_ETIMEOUT (the fields of that solve are invalid; the handle stays
+                             usable). One-shot: cleared by that launch. 0: off. Needs MOND_OPT_PIPELINED 1
+                             and no graph replay. */
   MOND_OPT_CYCLE_MEAN = 9,    /* value 1: a solve with n_iter >= 2 (plain or warm-started, not incremental)
                              takes as its potential the mean of the potentials of its last two iterations'
                              curl-free steps, phi^ = (phi^_{K-1} + phi^_K)/2. Near zeros of the field the

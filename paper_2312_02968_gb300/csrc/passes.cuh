@@ -687,9 +687,11 @@ __global__ void __launch_bounds__(NT) k_zpass(ZArgs a) {
 }  // namespace passes
 
 // ===========================================================================
-// Staged y-pass (the bounded-wait tests; the passes of a solve are those of
-// regpass.cuh): persistent CTAs stream tiles through a two-stage shared-memory
-// ring. One thread issues TMA tile loads (completion on an
+// Staged y-pass: the one kernel that waits on the device (for its TMA copies),
+// kept for the tests of a bounded wait that runs out. No solve launches it but
+// with MOND_OPT_TEST_LOST_LOAD: its passes are those of regpass.cuh, which wait
+// for nothing but the kernel before. Persistent CTAs stream tiles through a
+// two-stage shared-memory ring. One thread issues TMA tile loads (completion on an
 // mbarrier) for tile i+1 and TMA stores of tile i-1 while all threads
 // transform tile i, so HBM traffic overlaps the shared-memory FFT.
 // ===========================================================================

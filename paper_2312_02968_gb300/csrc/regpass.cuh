@@ -265,11 +265,21 @@ __device__ __forceinline__ void istep1(float2* v, const float2* sm, int j, const
 
 // ---------------------------------------------------------------------------
 // y-passes
+//
+// Folded: away from the Nyquist planes the curl-free projection k (k.g) A is the
+// gradient of one scalar, and so are the final and Newton operators. The y-pass
+// before such a z-pass folds the x and y components into s = kx gx^ + ky gy^
+// (component 0; component 2 keeps gz^), the z-pass takes the two and returns the
+// scalar u and the z component, and the y-pass after it unfolds u into kx u and
+// ky u ahead of its transform. On the column kx = N/2 and the row ky = N/2 the
+// Nyquist rule of the projection splits the axes into two sets, so that gx^ and
+// gy^ stay apart there (components 0 and 1) and the z-pass works on three
+// components; for Newton, kappa vanishes there and everything is folded.
 // ---------------------------------------------------------------------------
 enum YKind {
   Y_FWD = 0,       // plain, components c0 .. c0 + nplain - 1
   Y_INV = 1,
-  Y_FOLD = 2,      // forward: s = kx gx^ + ky gy^ into component 0 (see passes.cuh), then the plain components
+  Y_FOLD = 2,      // forward: s = kx gx^ + ky gy^ into component 0, then the plain components
   Y_CURL = 3,      // inverse after the curl-free z-pass: kx u, ky u (kt = k)
   Y_GRADN = 4,     // inverse after the final z-pass: kappa_x u, kappa_y u (kt = kappa)
   Y_GRAD = 5       // inverse after the Newton z-pass: as Y_GRADN, nothing apart on the Nyquist planes
