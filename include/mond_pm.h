@@ -130,7 +130,8 @@ enum {
   MOND_OPT_GRID_CAP = 11      /* value c > 0: the y/z passes, the deposit and the gather of a step
                              launch at most c CTAs (each working on several tiles), leaving the rest of the GPU to
                              kernels that run beside them (independent systems on their own streams,
-                             a batch); 0 (default): as many as fit the GPU. Same results. */
+                             a batch); 0 (default): a CTA per tile for the y/z passes, as many as are
+                             resident for the deposit and the gather. Same results. */
 };
 
 /* Per kernel class: launches, device time between the events around each

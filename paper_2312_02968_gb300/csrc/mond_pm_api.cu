@@ -299,10 +299,10 @@ struct mond_pm : StepState {
     float* dgN = nullptr;
   } inc;
   int keep_phi = 0, track_dh = 0, use_graph = 0, timing = 0, pipelined = 1;
-  int lost_tile = -1;  // MOND_OPT_TEST_LOST_LOAD: tile of the next pipelined y-pass whose copy is not issued
+  int lost_tile = -1;  // MOND_OPT_TEST_LOST_LOAD: tile of the staged y-pass whose copy is not issued (one-shot)
   int cycle_mean = 0;  // MOND_OPT_CYCLE_MEAN
   int fold = 1;        // MOND_OPT_FOLD (used where the pipelined passes run and the size allows it)
-  int grid_cap = 0;    // MOND_OPT_GRID_CAP: CTAs of a persistent kernel at most (0: all that fit)
+  int grid_cap = 0;    // MOND_OPT_GRID_CAP: CTAs of a y/z pass, the deposit and the gather at most (0: no cap)
   // mond_pm_step_host: the velocities go in on a copy stream of their own while
   // the deposit and the solve run; the gather waits for them (vel_wait)
   cudaStream_t copy_st = nullptr;

@@ -19,7 +19,11 @@ constexpr int CHUNK = 1024;   // default particles per work item (runtime: the a
 // 0.90 / 0.75, 0.86 / 0.70, 0.83 / 0.73, 0.82 / 0.75, 0.82 / 0.83, 0.79 / 1.02
 // ms for 1e6 particles of an isothermal sphere on 256^3 (sigma 1.5), and 0.20 /
 // 0.16, 0.18 / 0.14, 0.17 / 0.13, 0.17 / 0.13, 0.16 / 0.14, 0.20 / 0.16 ms for
-// 4e5 of a Plummer sphere on 192^3 (sigma 1).
+// 4e5 of a Plummer sphere on 192^3 (sigma 1). At sigma 2, 8, 16 and 24: 1.73 /
+// 1.35, 1.69 / 1.30, 1.74 / 1.34 ms for 1e6 on 256^3; only where all tiles hold
+// about as many as the limit does it matter (6e4 uniform on 128^3, 15 a
+// tile: sigma 2 0.40 / 0.32, 0.49 / 0.41, 0.60 / 0.51 ms, sigma 1 0.090
+// / 0.078, 0.076 / 0.067, 0.075 / 0.065).
 constexpr int SPARSE = 16;
 constexpr int SMS = 152;      // SMs of the GPU
 constexpr int QHALF = 32768;  // offset quantisation: q = round(offset * 2^16) + 32768

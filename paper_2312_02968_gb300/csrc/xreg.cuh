@@ -159,7 +159,8 @@ __device__ __forceinline__ void fwd_pair(const float2* s, int m, const float2* t
     const float2 pb = z ? b[A0 - 1 - r] : a[A0 - 1 - r];
     float2 xa = post1(a[r], pa, tw[j0 + A1 * r]);
     if (r == 0 && z) {
-      // k = 0 and k = H from Z[0]; the pad columns are zero
+      // k = 0 and k = H from Z[0]; the pad columns past H are left as they are
+      // (read with their neighbours by wide copies, used by nothing)
       xa = make_float2(a[0].x + a[0].y, 0.f);
       g[H] = make_float2(a[0].x - a[0].y, 0.f);
     }
