@@ -550,12 +550,26 @@ __global__ void __launch_bounds__(256) k_gelu_bwd(const float4* __restrict__ z, 
   }
 }
 
-__global__ void k_sumsq(const float* t, int64_t n, double* out) {
-  double s = 0.0;
+// Sum over the CTA (of 256 threads) of r, added to out by its first thread.
+__device__ __forceinline__ void block_add(double r, double* out) {
+  __shared__ double part[8];
+  for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = r;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) r += part[w];
+    atomicAdd(out, r);
+  }
+}
+
+// Sum of the squares in FP64, added to out: few floats, or a misaligned array.
+__global__ void __launch_bounds__(256) k_sumsq(const float* t, int64_t n, double* out) {
+  kernel_wait();
+  t = after_wait(t);
+  double r = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    s += (double)t[i] * t[i];
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
+    r += (double)t[i] * t[i];
+  block_add(r, out);
 }
 
 __global__ void k_loss(const float* y, const float* t, float* dy, int64_t n, const double* tnorm, float weight,
@@ -578,23 +592,22 @@ __global__ void k_loss(const float* y, const float* t, float* dy, int64_t n, con
   if ((threadIdx.x & 31) == 0) atomicAdd(loss, s * inv * weight);
 }
 
-// Sum of the squares of floats (16-byte aligned), added to out. Bound by the
-// read: every product is exact as two floats and the sums are compensated (FP32
-// pairs, about 48 bits), as this GPU's FP64 rate is a 64th of its FP32 rate. A
-// thread whose values leave the range where that is exact enough (past 1e18 in
-// size, all below 1e-12, infinities, NaNs) sums them in FP64. Over many
-// threads the pairs' roundings average out: against the exact sum 1e-15 (rms)
-// for 98304 floats and 1.2e-15 for 5e6, where FP64 sums and an unordered add
-// per warp are off by 1.5e-15 and 6.5e-15. Below PAIRS vectors they do not
-// (1.5e-15 against 2e-16 for 64 floats) and all is FP64, one vector a thread.
-// 134e6 floats: 252 us (FP64 sums) -> 96 us, 5.6 TB/s; 786432 floats: 40 -> 6 us.
-constexpr int64_t PAIRS = 16384;
+// The same of many floats (16-byte aligned). Bound by the read: every product is
+// exact as two floats and the sums are compensated (FP32 pairs, about 48 bits),
+// as this GPU's FP64 rate is a 64th of its FP32 rate. A thread whose values
+// leave the range where that is exact enough (past 1e18 in size, all below
+// 1e-12, infinities, NaNs) sums them in FP64. Over many threads the pairs'
+// roundings average out: against the exact sum 1e-15 (rms) for 98304 floats and
+// 1.2e-15 for 5e6, where FP64 sums with an unordered add per warp are off by
+// 1.5e-15 and 6.5e-15. For few they do not (1.5e-15 against 2e-16 for 64
+// floats): below PAIRS floats the sum is k_sumsq's. 134e6 floats: 252 us (FP64
+// sums) -> 96 us, 5.6 TB/s; 786432 floats: 40 -> 6 us.
+constexpr int64_t PAIRS = 65536;
 __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, int64_t n4, const float* __restrict__ tail,
                                                   int ntail, double* out) {
   kernel_wait();
   t = after_wait(t);
   tail = after_wait(tail);
-  __shared__ double part[8];
   float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f}, top = 0.f;
   auto add = [&](int k, float x) {
     const float p = __fmul_rn(x, x), e = __fmaf_rn(x, x, -p);
@@ -604,21 +617,18 @@ __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, 
     top = fmaxf(top, fabsf(x));
   };
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool pairs = n4 >= PAIRS;
-  if (pairs) {
 #pragma unroll 4
-    for (int64_t i = i0; i < n4; i += stride) {
-      const float4 x = *(t + i);
-      add(0, x.x);
-      add(1, x.y);
-      add(2, x.z);
-      add(3, x.w);
-    }
-    if (i0 < ntail) add(0, tail[i0]);
+  for (int64_t i = i0; i < n4; i += stride) {
+    const float4 x = *(t + i);
+    add(0, x.x);
+    add(1, x.y);
+    add(2, x.z);
+    add(3, x.w);
   }
+  if (i0 < ntail) add(0, tail[i0]);
   double r = 0.0;
   const float sum = (s[0] + s[1]) + (s[2] + s[3]);
-  if (pairs && isfinite(sum) && top < 1e18f && (top == 0.f || top > 1e-12f)) {
+  if (isfinite(sum) && top < 1e18f && (top == 0.f || top > 1e-12f)) {
     // the four sums as one float pair, then one FP64 addition a thread
 #pragma unroll
     for (int k = 1; k < 4; k++) {
@@ -634,13 +644,7 @@ __global__ void __launch_bounds__(256) k_gradnorm(const float4* __restrict__ t, 
     }
     if (i0 < ntail) r += (double)tail[i0] * tail[i0];
   }
-  for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = r;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; w++) r += part[w];
-    atomicAdd(out, r);
-  }
+  block_add(r, out);
 }
 
 struct AdamArgs {
@@ -1044,12 +1048,12 @@ unsigned grid_stride(int64_t n) {
 
 // *out += the sum of the squares of t.
 void sumsq(const float* t, int64_t n, double* out, cudaStream_t st) {
-  if (aligned16(t))
-    // pairs: eight vectors a thread at least, as a thread ends with FP64 sums
-    launch_early(k_gradnorm, grid_stride(n / 4 >= PAIRS ? (n + 31) / 32 : (n + 3) / 4), TB, 0, st, reinterpret_cast<const float4*>(t), n / 4,
+  if (aligned16(t) && n >= PAIRS)
+    // eight vectors a thread at least: a thread ends with FP64 sums
+    launch_early(k_gradnorm, grid_stride((n + 31) / 32), TB, 0, st, reinterpret_cast<const float4*>(t), n / 4,
                  t + n / 4 * 4, (int)(n % 4), out);
   else
-    k_sumsq<<<grid_stride(n), TB, 0, st>>>(t, n, out);
+    launch_early(k_sumsq, grid_stride((n + 3) / 4), TB, 0, st, t, n, out);
 }
 
 // The plane kernels may need more than the default 48 KB of shared memory.
