@@ -207,8 +207,8 @@ int mond_pm_set_density(mond_pm_t h, const float* rho);
  * curl-free projection and the acceleration mesh a = -grad_FD phi is formed.
  * n_iter = 0 gives the Newtonian solve (a = g_N). warm: MOND_WARM_NONE
  * (H = 0), MOND_WARM_PREV (H of the previous solve), MOND_WARM_GUESS
- * (H_guess: device float32, 3 planes; it is projected onto its
- * divergence-free part first) or MOND_WARM_GUESS_RAW (H_guess used as
+ * (H_guess: device float32, 3 planes, 8-byte aligned; it is projected onto
+ * its divergence-free part first) or MOND_WARM_GUESS_RAW (H_guess used as
  * given, once: the H state is left as it was). With MOND_WARM_PREV or
  * MOND_WARM_GUESS the last iteration also completes the H update so the next
  * solve can start from it. The Newtonian field is computed once
@@ -248,7 +248,7 @@ int mond_pm_set_increment_workspace(mond_pm_t h, void* ws, size_t bytes);
 /* Node-smoothed acceleration: the periodic discrete convolution of the
  * acceleration mesh with the ball-truncated Gaussian of Eq. gi, i.e. the force
  * Eq. gi gives a particle sitting exactly on each pixel centre. Written to
- * accel_mesh_out (device float32, 3 planes) when non-NULL and kept for
+ * accel_mesh_out (device float32, 3 planes, 8-byte aligned) when non-NULL and kept for
  * mond_pm_get_field(MOND_FIELD_SMOOTH). */
 int mond_pm_smooth(mond_pm_t h, float* accel_mesh_out);
 

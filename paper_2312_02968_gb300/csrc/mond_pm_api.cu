@@ -1437,6 +1437,7 @@ int mond_pm_solve_field(mond_pm_t h, int n_iter, int warm, const float* H_guess)
   if (warm < 0 || warm > 4) return fail(h, MOND_EINVAL, "bad warm mode %d", warm);
   if ((warm == MOND_WARM_GUESS || warm == MOND_WARM_GUESS_RAW) && !H_guess)
     return fail(h, MOND_EINVAL, "a guess warm start needs H_guess");
+  if (H_guess && ((uintptr_t)H_guess & 7)) return fail(h, MOND_EINVAL, "H_guess must be 8-byte aligned");
   if (warm != MOND_WARM_NONE && n_iter == 0) return fail(h, MOND_EINVAL, "a warm start needs n_iter >= 1");
   if (warm == MOND_WARM_INCREMENT) {
     if (const char* why = inc_unready(h)) return fail(h, MOND_ESTATE, "incremental solve: %s", why);
@@ -1449,6 +1450,7 @@ int mond_pm_smooth(mond_pm_t h, float* accel_mesh_out) {
   Range nvtx_range("mond_pm_smooth");
   if (!h) return MOND_EINVAL;
   if (!h->have_solve) return fail(h, MOND_ESTATE, "smooth before solve_field");
+  if ((uintptr_t)accel_mesh_out & 7) return fail(h, MOND_EINVAL, "accel_mesh_out must be 8-byte aligned");
   int rk = ensure_khat(h);
   if (rk) return rk;
   passes::XArgs xf{};

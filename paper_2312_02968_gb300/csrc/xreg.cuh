@@ -264,8 +264,8 @@ __global__ void __launch_bounds__(32 * WARPS, ncomp_of(MODE) == 3 ? xctas(N) : 1
     const uint32_t rb = (uint32_t)(X::LW * N * sizeof(float));
     const int64_t o = lane * P3 + ((int64_t)blockIdx.x * WARPS + warp) * X::LW * N;
     if constexpr (MODE == X_NU || MODE == X_MU || MODE == X_NU_REAL) tma::prefetch_l2(a.gN + o, rb);
-    if constexpr (MODE == X_NU_FIRST || MODE == X_NU_REAL)
-      if (a.H0) tma::prefetch_l2(a.H0 + o, rb);
+    if constexpr (MODE == X_NU_FIRST || MODE == X_NU_REAL)  // a caller's guess may lie off the prefetch's 16 bytes
+      if (a.H0 && (reinterpret_cast<uintptr_t>(a.H0) & 15) == 0) tma::prefetch_l2(a.H0 + o, rb);
     if constexpr (MODE == X_NU)
       if (a.Hs_out && a.red) tma::prefetch_l2(a.Hs_out + o, rb);
   }
